@@ -1385,10 +1385,10 @@ int diag_grid(ann_ctx *c, int M)
     if (st) return st;
     size_t n = (size_t)c->P.n, MM = (size_t)M * M;
     cudaError_t e = ensure(c, c->d_grid, 5 * MM * sizeof(double));
-    if (!e) e = ensure(c, c->d_off, n * sizeof(float2));
+    if (!e) e = ensure(c, c->d_off, n * sizeof(float2) + sizeof(unsigned));   // and the excursion word
     if (!e) e = ensure(c, c->d_fld, n * sizeof(float4));
-    if (!e) e = enqueue_grid(c->P, c->b, src, M, (float2 *)c->d_off.p, (float4 *)c->d_fld.p, (double *)c->d_grid.p,
-                             c->stream);
+    if (!e) e = enqueue_grid(c->P, c->b, src, M, (float2 *)c->d_off.p, (float4 *)c->d_fld.p,
+                             (unsigned *)((float2 *)c->d_off.p + n), (double *)c->d_grid.p, c->stream);
     if (!e) e = cudaStreamSynchronize(c->stream);
     if (e) return cuda_fail(c, e, "gridding");
     c->grid_M = M;
@@ -1500,9 +1500,10 @@ int ann_vorticity_correlation(ann_ctx *c, int32_t M, int32_t all_origins, double
     if (!c || !C || (all_origins != 0 && all_origins != 1)) return ANN_ERR_INVALID_ARG;
     int st = diag_grid(c, M);
     if (st) return st;
-    cudaError_t e = ensure(c, c->d_out, (size_t)std::max(nshell_of(M), M / 2 + 1) * sizeof(double));
-    if (!e) e = enqueue_correlation(M, c->prm.L, (const double *)c->d_grid.p, all_origins, (double *)c->d_out.p,
-                                    c->stream);
+    // C (M/2 + 1 values), then the centre row's vorticity (M)
+    cudaError_t e = ensure(c, c->d_out, (size_t)std::max(nshell_of(M), M / 2 + 1 + M) * sizeof(double));
+    double *dC = (double *)c->d_out.p;
+    if (!e) e = enqueue_correlation(M, c->prm.L, (const double *)c->d_grid.p, all_origins, dC, dC + M / 2 + 1, c->stream);
     if (!e) e = cudaMemcpyAsync(C, c->d_out.p, (size_t)(M / 2 + 1) * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
     if (!e) e = cudaStreamSynchronize(c->stream);
     if (e) return cuda_fail(c, e, "ann_vorticity_correlation");

@@ -193,12 +193,15 @@ struct DiagSrc {
     const float4 *u4;                   // (ux, uy, q11, q12) records when not null
 };
 // grid: 5 x M x M doubles (ux, uy, q11, q12, Shepard weight sum), [field][iy][ix]
+// off, fld: scratch of n values; out: scratch of one word
 cudaError_t enqueue_grid(const DevParams &P, const Bufs &b, DiagSrc src, int M, float2 *off, float4 *fld,
-                         double *grid, cudaStream_t s);
+                         unsigned *out, double *grid, cudaStream_t s);
 cudaError_t enqueue_twiddles(int M, double2 *tw, cudaStream_t s);
 cudaError_t enqueue_spectrum(int M, const double *grid, double2 *z, double2 *zt, const double2 *tw,
                              const int *shell_off, const int *shell_modes, int nshell, double *E, cudaStream_t s);
-cudaError_t enqueue_correlation(int M, double L, const double *grid, int all_origins, double *C, cudaStream_t s);
+// om: scratch of M doubles (the centre row's vorticity)
+cudaError_t enqueue_correlation(int M, double L, const double *grid, int all_origins, double *C, double *om,
+                                cudaStream_t s);
 cudaError_t enqueue_defects(int M, const double *grid, signed char *map, unsigned long long *counts, cudaStream_t s);
 cudaError_t enqueue_mixing(const DevParams &P, const Bufs &b, const unsigned char *colors, int G, int S,
                            unsigned *cnt, cudaStream_t s);
