@@ -1,6 +1,6 @@
 // C-ABI of the SPH active-nematic solver: context, device buffers, CUDA-graph step, I/O.
 #include "../../include/ann.h"
-#include "ann_internal.cuh"
+#include "ann_device.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -554,6 +554,23 @@ bool field_of(ann_ctx *c, int f, Field &out)
     }
 }
 
+// A loaded coordinate in [0, L), never -0.  Nearly every one is there already, which two integer
+// comparisons tell: the FP64 comparisons and additions below (2 a cycle and SM) would bound the load.
+__device__ __forceinline__ double reinsert(double x, const DevParams &P)
+{
+    if (in_box(x, P.bitsL)) return x;
+    if (x < -P.L || x >= 2.0 * P.L) x = x - floor(x / P.L) * P.L;
+    if (x < 0.0) x += P.L;
+    if (x >= P.L) x -= P.L;
+    return x + 0.0;
+}
+
+// FP64 finiteness on the bit pattern.
+__device__ __forceinline__ bool finite_d(double x)
+{
+    return (__double_as_longlong(x) & 0x7ff0000000000000ll) != 0x7ff0000000000000ll;
+}
+
 // ann_set_state's load: the state as the context stores it (FP64 positions, FP32 fields, the
 // density as its deviation), re-inserted into the box as ann_set_particles does.
 __global__ void k_load_state(DevParams P, Bufs b, const double *x, const double *y, const float *ux,
@@ -563,20 +580,16 @@ __global__ void k_load_state(DevParams P, Bufs b, const double *x, const double 
     if (i >= P.n) return;
     double xx = x[i], yy = y[i];
     const float d = drho ? drho[i] : 0.f;
-    if (!(isfinite(xx) && isfinite(yy) && isfinite(ux[i]) && isfinite(uy[i]) && isfinite(q11[i]) &&
+    if (!(finite_d(xx) && finite_d(yy) && isfinite(ux[i]) && isfinite(uy[i]) && isfinite(q11[i]) &&
           isfinite(q12[i]) && isfinite(d) && d > -1.f)) {
         atomicOr(b.err, EB_NONFINITE);
         xx = 0.0;
         yy = 0.0;
     }
-    if (xx < -P.L || xx >= 2.0 * P.L) xx = xx - floor(xx / P.L) * P.L;
-    if (yy < -P.L || yy >= 2.0 * P.L) yy = yy - floor(yy / P.L) * P.L;
-    if (xx < 0.0) xx += P.L;
-    if (xx >= P.L) xx -= P.L;
-    if (yy < 0.0) yy += P.L;
-    if (yy >= P.L) yy -= P.L;
-    b.sx[i] = xx + 0.0;
-    b.sy[i] = yy + 0.0;
+    xx = reinsert(xx, P);
+    yy = reinsert(yy, P);
+    b.sx[i] = xx;
+    b.sy[i] = yy;
     b.sux[i] = ux[i];
     b.suy[i] = uy[i];
     b.sq11[i] = q11[i];
@@ -592,20 +605,16 @@ __global__ void k_load_state(DevParams P, Bufs b, const double *x, const double 
 __device__ __forceinline__ void store_slot(const DevParams &P, const Bufs &b, int g, int id, double xx, double yy,
                                           float ux, float uy, float q11, float q12, float d, float a0, float a1)
 {
-    if (!(isfinite(xx) && isfinite(yy) && isfinite(ux) && isfinite(uy) && isfinite(q11) && isfinite(q12) &&
+    if (!(finite_d(xx) && finite_d(yy) && isfinite(ux) && isfinite(uy) && isfinite(q11) && isfinite(q12) &&
           isfinite(d) && d > -1.f && isfinite(a0) && isfinite(a1))) {
         atomicOr(b.err, EB_NONFINITE);
         xx = 0.0;
         yy = 0.0;
     }
-    if (xx < -P.L || xx >= 2.0 * P.L) xx = xx - floor(xx / P.L) * P.L;
-    if (yy < -P.L || yy >= 2.0 * P.L) yy = yy - floor(yy / P.L) * P.L;
-    if (xx < 0.0) xx += P.L;
-    if (xx >= P.L) xx -= P.L;
-    if (yy < 0.0) yy += P.L;
-    if (yy >= P.L) yy -= P.L;
-    b.sx[g] = xx + 0.0;
-    b.sy[g] = yy + 0.0;
+    xx = reinsert(xx, P);
+    yy = reinsert(yy, P);
+    b.sx[g] = xx;
+    b.sy[g] = yy;
     b.sux[g] = ux;
     b.suy[g] = uy;
     b.sq11[g] = q11;
