@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(256) k_grid(DevParams P, Bufs b, int M, const 
 }
 
 // ------------------------------------------------------------------------------------------------
-// FFT (FP64, radix 2, M a power of two).  z = ux + i uy is transformed along rows, transposed and
+// FFT (FP64, radix 4, M a power of two).  z = ux + i uy is transformed along rows, transposed and
 // transformed along rows again; |Z|^2 is symmetric under the transposition as far as the shells
 // are concerned (|k| depends on kx^2 + ky^2).  E_n = 1/2 sum_{|k| -> n} |Z(k)|^2 / M^4 equals
 // 1/2 sum (|ux_hat|^2 + |uy_hat|^2) with u_hat = fft2(u) / M^2, because Z(k) = Ux(k) + i Uy(k)
@@ -128,30 +128,86 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b)
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// One row per block: bit-reversed load into shared memory, log2 M butterfly stages, natural store.
-// PACK: the input is the real grid pair (ux, uy) packed as ux + i uy.
-template <bool PACK>
-__global__ void k_fft_rows(int M, int logM, const double2 *in, const double *gx, const double *gy, double2 *out,
-                           const double2 *tw)
+__device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+
+// p = a + w b, m = a - w b (six operations: m = 2a - p)
+__device__ __forceinline__ void butterfly(double2 a, double2 b, double2 w, double2 &p, double2 &m)
 {
-    extern __shared__ double2 row[];
-    size_t base = (size_t)blockIdx.x * M;
-    for (int i = threadIdx.x; i < M; i += blockDim.x) {
-        int r = (int)(__brev((unsigned)i) >> (32 - logM));
-        row[r] = PACK ? make_double2(gx[base + i], gy[base + i]) : in[base + i];
+    p.x = fma(w.x, b.x, fma(-w.y, b.y, a.x));
+    p.y = fma(w.x, b.y, fma(w.y, b.x, a.y));
+    m.x = fma(2.0, a.x, -p.x);
+    m.y = fma(2.0, a.y, -p.y);
+}
+
+// One row per block of M/4 threads: radix-4 passes of the self-sorting (Stockham) FFT, four points
+// a thread in registers, one exchange through shared memory between passes; a last radix-2 pass when
+// log2 M is odd.  Pass with sub-transforms of L points: thread j takes points j + r M/4, multiplies by
+// exp(-2 pi i r k / 4L), k = j mod L, and writes 4 (j - k) + k + r L.  The first pass reads and the
+// last writes global memory (coalesced).  The work is FP64 issue (2 a cycle and SM): 112 operations
+// a thread of M = 1024 (16 in the first pass, whose factors are 1, and 24 in each other) against the
+// 160 a thread would have in radix-2 passes; M = 1024: 79 us a dimension (ncu,
+// cold caches), radix 2 took 92.  The
+// exchange buffer is padded by an element in four, which keeps the stride-4 writes of the first pass
+// free of bank conflicts.  PACK: the input is the real grid pair (ux, uy) packed as ux + i uy.
+__host__ __device__ constexpr int fft_pad(int i) { return i + (i >> 2); }
+
+template <bool PACK>
+__global__ void __launch_bounds__(512) k_fft_rows(int M, int logM, const double2 *in, const double *gx, const double *gy,
+                                                  double2 *out, const double2 *tw)
+{
+    extern __shared__ double2 sm[];
+    const size_t base = (size_t)blockIdx.x * M;
+    const int Q = M / 4, j = threadIdx.x;
+    double2 *buf = sm;
+    double2 x[4];
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        const size_t i = base + j + r * Q;
+        x[r] = PACK ? make_double2(gx[i], gy[i]) : in[i];
     }
-    __syncthreads();
-    for (int half = 1; half < M; half <<= 1) {
-        int stride = M / (2 * half);
-        for (int t = threadIdx.x; t < M / 2; t += blockDim.x) {
-            int pos = t % half, i = (t / half) * 2 * half + pos, j = i + half;
-            double2 a = row[i], w = cmul(row[j], tw[pos * stride]);
-            row[i] = make_double2(a.x + w.x, a.y + w.y);
-            row[j] = make_double2(a.x - w.x, a.y - w.y);
+    int L = 1;
+    for (; 4 * L <= M; L *= 4) {
+        const int k = j & (L - 1), st = Q / L;   // factor r is exp(-2 pi i r k st / M)
+        double2 a, b, c, d;   // a, b = x0 +- w2 x2, c, d = w1 x1 +- w3 x3
+        if (L == 1) {
+            a = cadd(x[0], x[2]);
+            b = csub(x[0], x[2]);
+            c = cadd(x[1], x[3]);
+            d = csub(x[1], x[3]);
+        } else {
+            const int i3 = 3 * k * st;   // up to 3/4 M: the table holds half a turn
+            double2 w3 = tw[i3 < M / 2 ? i3 : i3 - M / 2];
+            if (i3 >= M / 2) w3 = make_double2(-w3.x, -w3.y);
+            butterfly(x[0], x[2], tw[2 * k * st], a, b);
+            butterfly(cmul(x[1], tw[k * st]), x[3], w3, c, d);
         }
+        x[0] = cadd(a, c);
+        x[2] = csub(a, c);
+        x[1] = make_double2(b.x + d.y, b.y - d.x);   // b - i d
+        x[3] = make_double2(b.x - d.y, b.y + d.x);
+        const int o = 4 * (j - k) + k;
+        if (4 * L == M) {   // done: o = j
+#pragma unroll
+            for (int r = 0; r < 4; r++) out[base + j + r * Q] = x[r];
+            return;
+        }
+#pragma unroll
+        for (int r = 0; r < 4; r++) buf[fft_pad(o + r * L)] = x[r];
         __syncthreads();
+        if (8 * L == M) break;   // a radix-2 pass is left
+#pragma unroll
+        for (int r = 0; r < 4; r++) x[r] = buf[fft_pad(j + r * Q)];
+        buf = buf == sm ? sm + fft_pad(M) : sm;   // the next pass writes the other buffer: one barrier a pass
     }
-    for (int i = threadIdx.x; i < M; i += blockDim.x) out[base + i] = row[i];
+#pragma unroll
+    for (int r = 0; r < 2; r++) {   // L = M/2: two of the M/2 pairs a thread
+        const int i = j + r * Q;
+        double2 p, m;
+        butterfly(buf[fft_pad(i)], buf[fft_pad(i + M / 2)], tw[i], p, m);
+        out[base + i] = p;
+        out[base + i + M / 2] = m;
+    }
 }
 
 __global__ void k_transpose(int M, const double2 *in, double2 *out)
@@ -364,8 +420,8 @@ cudaError_t enqueue_spectrum(int M, const double *grid, double2 *z, double2 *zt,
 {
     int logM = 0;
     while ((1 << logM) < M) logM++;
-    int th = M / 2 < 512 ? M / 2 : 512;
-    size_t smem = sizeof(double2) * (size_t)M;
+    const int th = M / 4;   // 2 (M = 8) to 512
+    size_t smem = sizeof(double2) * 2 * (size_t)fft_pad(M);
     cudaError_t e = cudaFuncSetAttribute(k_fft_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (!e) e = cudaFuncSetAttribute(k_fft_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e) return e;
