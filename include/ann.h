@@ -604,8 +604,8 @@ int ann_velocity_moments_noalloc(const float *ux, const float *uy, const float *
  * corrected Laplacian is the scalar form with factor 2 per component; the viscous term of Eq. (23)
  * carries 2 (d + 2) nu = 10 nu.  Paper momentum mode only, no elastic stress.  A periodic cube of
  * side L; cells of side >= 3h (1 + 0.05), at least 3 per side (L >= 9.45 h: 13 particles a side at
- * h = 1.3 dx).  Candidate lists (every j within 3h (1 + 0.05), rebuilt with a re-sort when a
- * particle has moved 0.05 x 3h / 2) hold at most 576, neighbour lists ANN3_MAX_NEIGHBORS (~250 at
+ * h = 1.3 dx).  Candidate lists (every j within 3h (1 + 0.02), rebuilt with a re-sort when a
+ * particle has moved 0.02 x 3h / 2) hold at most 576, neighbour lists ANN3_MAX_NEIGHBORS (~250 at
  * h = 1.3 dx).  FP64 positions; pair differences are taken
  * in FP64 and everything else runs in FP32.  The step order is that of the 2D step (modified
  * Euler predictor, search, volumes, correction tensor, continuity, density filter and equation of
