@@ -170,6 +170,17 @@ int validate(const ann_params *p, std::string &why)
     return ANN_OK;
 }
 
+// Lanes per particle of passes A to D: as many (1, 2, 4 or 8) as keep the blocks at two per SM.  Every lane
+// more stages the halo and runs the epilogue once more, so lanes pay only where SMs would idle.  Measured
+// (us per step with 1 / 2 / 4 / 8 lanes): 16 tiles (64^2) 59 / 47 / 46 / 44, 64 tiles (128^2) 60 / 49 / 49 /
+// 58, 144 tiles (180^2) 60 / 58 / 64 / 80, 256 tiles (256^2) 72 / 77 / 89 / 122.
+int lanes_for(int tiles)
+{
+    int lanes = 8;
+    while (lanes > 1 && tiles * lanes > 304) lanes /= 2;   // 152 SMs
+    return lanes;
+}
+
 DevParams make_dev(const ann_params &p)
 {
     DevParams d{};
@@ -177,6 +188,7 @@ DevParams make_dev(const ann_params &p)
     d.nc = cells_per_side(p);
     d.ncell = d.nc * d.nc;
     d.tiles = (d.nc + TILE - 1) / TILE;
+    d.lanes = lanes_for(d.tiles * d.tiles);
     d.apd = p.apd;
     d.conservative = p.momentum_mode == ANN_MOMENTUM_CONSERVATIVE;
     d.qnew = p.q_new_in_momentum;

@@ -50,6 +50,7 @@ enum : uint32_t {
 // Parameters in the form the kernels use (FP64 where positions are involved).
 struct DevParams {
     int n, nc, ncell, tiles;
+    int lanes;             // lanes per particle of passes A to D (1, 2, 4 or 8), by the tile count
     int apd, conservative, qnew, record, elastic;
     double L, cell, inv_cell, R2, dt_d, half_dt_d;
     double q;              // power-of-two grid of the "hi" coordinate part: cell / q in [2^12, 2^13)

@@ -54,69 +54,107 @@ __device__ __forceinline__ void add_crossing(const Bufs &b, int id, int kx, int 
 // Tile bookkeeping shared by the pair passes
 // ---------------------------------------------------------------------------------------------
 
+// Halo cells are numbered h = hy * HALO + hx whatever the tile's size; in a tile cut by the box (fewer
+// than TILE cells) the cells past its halo hold no slots.
 struct TileShared {
-    int off[NHC + 1];      // exclusive prefix of halo-cell particle counts (slots)
-    int start[NHC];        // first sorted index of each halo cell
-    int rowpre[TILE + 1];  // prefix of inner-row slot counts
+    int off[64];           // exclusive prefix of the halo cells' particle counts (slots); INT_MAX past off[NHC]
+    int4 cell[NHC];        // (first sorted index - first slot, bits of the floats hx and hy, -) of each halo cell
+    int4 rowpre;           // inner particles before row r = 0..3
+    int rowslot[TILE];     // slot of row r's first inner particle, less rowpre[r]
+    int Ni;                // inner particles
+    bool stop;             // an error has been raised: the block does nothing
 };
 
 struct Tile {
-    int cx0, cy0, wx, wy, HX, NH, H, Ni;
+    int H, Ni;   // slots, inner particles
 };
 
+__device__ __forceinline__ bool first_thread() { return (blockIdx.x | blockIdx.y | threadIdx.x) == 0; }
+
+// Set up by the block's first warp; blocks are a grid of tiles (x, y), LP blocks per tile along x (see
+// "Lanes per particle" below).  Everything a thread does per tile or per slot counts: with a search
+// loop and divisions per slot, and a prefix by one thread, set-up and staging were a third of the
+// instructions of a pass; now they are 200 of 2,150 to 2,900 per warp (512^2: A 27.7 -> 25.6 us, D 35.8 ->
+// 34.7).  False: an error has been raised, here (the halo does not fit) or before -- decided once for the
+// whole block, since another block may raise one at any time.
+template <int LP = 1>
 __device__ __forceinline__ bool tile_begin(const DevParams &P, const Bufs &b, TileShared &ts, Tile &T)
 {
-    int tx = blockIdx.x % P.tiles, ty = blockIdx.x / P.tiles;
-    T.cx0 = tx * TILE;
-    T.cy0 = ty * TILE;
-    T.wx = min(TILE, P.nc - T.cx0);
-    T.wy = min(TILE, P.nc - T.cy0);
-    T.HX = T.wx + 2;
-    T.NH = T.HX * (T.wy + 2);
-    int t = threadIdx.x;
-    if (t < T.NH) {
-        int hx = t % T.HX, hy = t / T.HX;
-        int c = wrapc(T.cy0 - 1 + hy, P.nc) * P.nc + wrapc(T.cx0 - 1 + hx, P.nc);
-        uint32_t s0 = b.cell_start[c], s1 = b.cell_start[c + 1];
-        ts.start[t] = (int)s0;
-        ts.off[t + 1] = (int)(s1 - s0);
-    }
-    __syncthreads();
-    if (t == 0) {
-        ts.off[0] = 0;
-        for (int h = 0; h < T.NH; h++) ts.off[h + 1] += ts.off[h];
-        int acc = 0;
-        ts.rowpre[0] = 0;
-        for (int r = 0; r < T.wy; r++) {
-            int row = (r + 1) * T.HX;
-            acc += ts.off[row + T.wx + 1] - ts.off[row + 1];
-            ts.rowpre[r + 1] = acc;
+    const int t = threadIdx.x;
+    if (t < 32) {
+        const int cx0 = (int)(blockIdx.x / LP) * TILE, cy0 = (int)blockIdx.y * TILE;
+        const int wx = min(TILE, P.nc - cx0), wy = min(TILE, P.nc - cy0);
+        const bool stop = stopped(b);
+        int first[2], cnt[2];   // halo cells t and t + 32
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            const int h = t + 32 * k, hx = h % HALO, hy = h / HALO;
+            first[k] = cnt[k] = 0;
+            if (h < NHC && hx < wx + 2 && hy < wy + 2) {
+                const int c = wrapc(cy0 - 1 + hy, P.nc) * P.nc + wrapc(cx0 - 1 + hx, P.nc);
+                const uint32_t s0 = b.cell_start[c], s1 = b.cell_start[c + 1];
+                first[k] = (int)s0;
+                cnt[k] = (int)(s1 - s0);
+            }
+        }
+        int v = cnt[0], u = cnt[1];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(FULL, v, o);
+            if (t >= o) v += x;
+        }
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {   // cells 32..35 sit in lanes 0..3
+            const int x = __shfl_up_sync(FULL, u, o);
+            if (t >= o) u += x;
+        }
+        u += __shfl_sync(FULL, v, 31);
+        const int all = __shfl_sync(FULL, u, NHC - 33);
+        ts.off[t] = v - cnt[0];
+        ts.off[t + 32] = t < NHC - 32 ? u - cnt[1] : (t == NHC - 32 ? all : 0x7fffffff);
+        ts.cell[t] = make_int4(first[0] - (v - cnt[0]), __float_as_int((float)(t % HALO)), __float_as_int((float)(t / HALO)), 0);
+        if (t < NHC - 32)
+            ts.cell[t + 32] = make_int4(first[1] - (u - cnt[1]), __float_as_int((float)((t + 32) % HALO)),
+                                        __float_as_int((float)((t + 32) / HALO)), 0);
+        __syncwarp();
+        if (t < TILE) {   // inner row t
+            const int lo = ts.off[(t + 1) * HALO + 1], hi = ts.off[(t + 1) * HALO + wx + 1];
+            const int c = t < wy ? hi - lo : 0;
+            int before = c;
+            int x = __shfl_up_sync(0xfu, before, 1);
+            if (t >= 1) before += x;
+            x = __shfl_up_sync(0xfu, before, 2);
+            if (t >= 2) before += x;
+            reinterpret_cast<int *>(&ts.rowpre)[t] = before - c;
+            ts.rowslot[t] = lo - (before - c);
+            if (t == TILE - 1) ts.Ni = before;
+        }
+        if (t == 0) {
+            if (!stop && all > HCAP) atomicOr(b.err, EB_HALO);
+            ts.stop = stop || all > HCAP;
         }
     }
     __syncthreads();
-    T.H = ts.off[T.NH];
-    T.Ni = ts.rowpre[T.wy];
-    return T.H <= HCAP;
+    T.H = ts.off[NHC];
+    T.Ni = ts.Ni;
+    return !ts.stop;
 }
 
 // Halo cell holding slot t (largest h with off[h] <= t).
-__device__ __forceinline__ int slot_cell(const TileShared &ts, int NH, int t)
+__device__ __forceinline__ int slot_cell(const TileShared &ts, int t)
 {
-    int lo = 0, hi = NH - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (ts.off[mid] <= t) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
+    int h = 0;
+#pragma unroll
+    for (int step = 32; step > 0; step >>= 1)
+        if (ts.off[h + step] <= t) h += step;
+    return h;
 }
 
 // Slot of the q-th particle of the tile's inner cells.
-__device__ __forceinline__ int inner_slot(const TileShared &ts, const Tile &T, int q)
+__device__ __forceinline__ int inner_slot(const TileShared &ts, int q)
 {
-    int r = 0;
-    while (r + 1 < T.wy && ts.rowpre[r + 1] <= q) r++;
-    return ts.off[(r + 1) * T.HX + 1] + (q - ts.rowpre[r]);
+    const int4 r = ts.rowpre;
+    return ts.rowslot[(q >= r.y) + (q >= r.z) + (q >= r.w)] + q;
 }
 
 // Sorted index and tile-local position (hi_x, hi_y, lo_x, lo_y) of slot t.  The halo cell offset
@@ -126,14 +164,15 @@ struct SlotInfo {
     float4 e;
 };
 
-__device__ __forceinline__ SlotInfo slot_info(const DevParams &P, const Bufs &b, const TileShared &ts,
-                                              const Tile &T, int t)
+template <bool REF = false>
+__device__ __forceinline__ SlotInfo slot_info(const DevParams &P, const Bufs &b, const TileShared &ts, int t)
 {
     SlotInfo s;
-    s.h = slot_cell(ts, T.NH, t);
-    s.g = ts.start[s.h] + (t - ts.off[s.h]);
-    float hx = (float)(s.h % T.HX), hy = (float)(s.h / T.HX);
-    float4 o = b.xi[s.g];
+    s.h = slot_cell(ts, t);
+    const int4 c = ts.cell[s.h];
+    s.g = c.x + t;
+    const float hx = __int_as_float(c.y), hy = __int_as_float(c.z);
+    const float4 o = REF ? b.xi_ref[s.g] : b.xi[s.g];
     s.e = make_float4(o.x + hx * P.cell_hi, o.y + hy * P.cell_hi, o.z + hx * P.cell_lo, o.w + hy * P.cell_lo);
     return s;
 }
@@ -441,7 +480,7 @@ constexpr int SMEM_A = HCAP * (16 + 4 + 1) + MAXV * PT * 2;
 template <bool FROM_REF>
 __global__ void __launch_bounds__(PT) k_pass_a_resort(DevParams P, Bufs b)
 {
-    if (stopped(b) || (!FROM_REF && !resorting(b))) return;
+    if (!FROM_REF && !resorting(b)) return;
     __shared__ TileShared ts;
     extern __shared__ __align__(16) unsigned char dsm[];
     float4 *pos = reinterpret_cast<float4 *>(dsm);
@@ -450,30 +489,24 @@ __global__ void __launch_bounds__(PT) k_pass_a_resort(DevParams P, Bufs b)
     uint16_t *lst = reinterpret_cast<uint16_t *>(sg + HCAP);
     unsigned char *shc = reinterpret_cast<unsigned char *>(lst + MAXV * PT);
     Tile T;
-    if (!tile_begin(P, b, ts, T)) {
-        if (threadIdx.x == 0) atomicOr(b.err, EB_HALO);
-        return;
-    }
+    if (!tile_begin(P, b, ts, T)) return;
     for (int t = threadIdx.x; t < T.H; t += PT) {
-        int h = slot_cell(ts, T.NH, t);
-        int g = ts.start[h] + (t - ts.off[h]);
-        float hx = (float)(h % T.HX), hy = (float)(h / T.HX);
-        float4 o = FROM_REF ? b.xi_ref[g] : b.xi[g];
-        pos[t] = make_float4(o.x + hx * P.cell_hi, o.y + hy * P.cell_hi, o.z + hx * P.cell_lo, o.w + hy * P.cell_lo);
-        sg[t] = g;
-        shc[t] = (unsigned char)h;
+        const SlotInfo s = slot_info<FROM_REF>(P, b, ts, t);
+        pos[t] = s.e;
+        sg[t] = s.g;
+        shc[t] = (unsigned char)s.h;
     }
     __syncthreads();
-    if (!FROM_REF && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(b.resorts, 1u);
+    if (!FROM_REF && first_thread()) atomicAdd(b.resorts, 1u);
     uint16_t *my = lst + threadIdx.x;   // this thread's list column, stride PT
     for (int q = threadIdx.x; q < T.Ni; q += PT) {
-        int si = inner_slot(ts, T, q);
-        int h = shc[si], hx = h % T.HX, hy = h / T.HX;
+        int si = inner_slot(ts, q);
+        const int h = shc[si];
         float4 pi = pos[si];
         int gi = sg[si];
         int cnt = 0;
         for (int oy = -1; oy <= 1; oy++) {
-            int row = (hy + oy) * T.HX + hx;
+            const int row = h + oy * HALO;
             int j0 = ts.off[row - 1], j1 = ts.off[row + 2];
             for (int j = j0; j < j1; j++) {
                 float2 pj = phi[2 * j];
@@ -549,6 +582,9 @@ __global__ void __launch_bounds__(PT) k_pass_a_resort(DevParams P, Bufs b)
 #ifndef ANN_MINB_D
 #define ANN_MINB_D 5
 #endif
+#ifndef ANN_MINB_L
+#define ANN_MINB_L 4
+#endif
 #ifndef ANN_PF_A
 #define ANN_PF_A 1
 #endif
@@ -563,22 +599,22 @@ __global__ void __launch_bounds__(PT) k_pass_a_resort(DevParams P, Bufs b)
 #endif
 #define ANN_BOUNDS(minb) __launch_bounds__(PT, (minb) > 0 ? (minb) : 1)
 #if ANN_MINB_A > 0
-#define BOUNDS_A ANN_BOUNDS(ANN_MINB_A)
+#define BOUNDS_A ANN_BOUNDS(LP > 1 ? ANN_MINB_L : ANN_MINB_A)
 #else
 #define BOUNDS_A __launch_bounds__(PT)
 #endif
 #if ANN_MINB_B > 0
-#define BOUNDS_B ANN_BOUNDS(ANN_MINB_B)
+#define BOUNDS_B ANN_BOUNDS(LP > 1 ? ANN_MINB_L : ANN_MINB_B)
 #else
 #define BOUNDS_B __launch_bounds__(PT)
 #endif
 #if ANN_MINB_C > 0
-#define BOUNDS_C ANN_BOUNDS(ANN_MINB_C)
+#define BOUNDS_C ANN_BOUNDS(LP > 1 ? ANN_MINB_L : ANN_MINB_C)
 #else
 #define BOUNDS_C __launch_bounds__(PT)
 #endif
 #if ANN_MINB_D > 0
-#define BOUNDS_D ANN_BOUNDS(ANN_MINB_D)
+#define BOUNDS_D ANN_BOUNDS(LP > 1 ? ANN_MINB_L : ANN_MINB_D)
 #else
 #define BOUNDS_D __launch_bounds__(PT)
 #endif
@@ -587,9 +623,34 @@ __global__ void __launch_bounds__(PT) k_pass_a_resort(DevParams P, Bufs b)
 // next PF words in flight while the current ones are processed: fn(byte offset of the slot,
 // candidate index, bit), bit = the entry's neighbour bit (nonzero iff the candidate is a neighbour).
 // Word m (candidates 4m .. 4m + 3) is loaded only when 4m < c.
-template <int PF, typename Fn>
+// With LP > 1 lanes per particle, lane l visits the words l, l + LP, ...
+template <int PF, int LP = 1, typename Fn>
 __device__ __forceinline__ void for_each_slot(const uint2 *list, int n, int gi, int c, Fn &&fn)
 {
+    if constexpr (LP > 1) {
+        const int l = threadIdx.x & (LP - 1);
+        const uint2 *p = list + (size_t)l * n + gi;
+        uint2 nxt = 4 * l < c ? __ldg(p) : make_uint2(0u, 0u);
+        for (int k = 4 * l; k < c; k += 4 * LP) {
+            const uint2 w = nxt;
+            p += (size_t)LP * n;
+            if (k + 4 * LP < c) nxt = __ldg(p);
+            if (k + 3 < c) {
+                fn((int)(w.x & SLOT_OFF_MASK), k, w.x & 1u);
+                fn((int)((w.x >> 16) & SLOT_OFF_MASK), k + 1, w.x & 0x10000u);
+                fn((int)(w.y & SLOT_OFF_MASK), k + 2, w.y & 1u);
+                fn((int)((w.y >> 16) & SLOT_OFF_MASK), k + 3, w.y & 0x10000u);
+            } else {
+                const unsigned long long w64 = ((unsigned long long)w.y << 32) | w.x;
+                for (int t = 0; k + t < c; t++) {
+                    const unsigned e = (unsigned)(w64 >> (16 * t));
+                    fn((int)(e & SLOT_OFF_MASK), k + t, e & 1u);
+                }
+            }
+        }
+        return;
+    }
+
     static_assert(PF >= 1 && PF <= 3, "prefetch distance");
     const uint2 *p = list + gi;
     uint2 r[PF + 1];   // r[0]: the current word, r[m]: word k/4 + m
@@ -617,10 +678,54 @@ __device__ __forceinline__ void for_each_slot(const uint2 *list, int n, int gi, 
 
 // Candidates of particle gi.  Beyond the support the clamped kernel gives W = F = 0 exactly, and
 // adding +0 or -0 leaves an FP32 sum unchanged, so sums over candidates equal sums over neighbours.
-template <int PF, typename Fn>
+template <int PF, int LP = 1, typename Fn>
 __device__ __forceinline__ void for_each_candidate(const DevParams &P, const Bufs &b, int gi, Fn &&fn)
 {
-    for_each_slot<PF>(b.vnbr, P.n, gi, b.vcnt[gi], fn);
+    for_each_slot<PF, LP>(b.vnbr, P.n, gi, b.vcnt[gi], fn);
+}
+
+// Lanes per particle (P.lanes: 1, 2, 4 or 8, the template argument LP of the passes).  A box of few
+// tiles leaves the GPU idle with one block per tile and one thread per particle: 64^2 has 16 tiles for
+// 152 SMs, and a thread's walk of 46 candidates is most of a pass.  There LP blocks share a tile (each
+// stages the whole halo and takes PT / LP of its particles) and LP lanes a particle's candidate words.
+template <int LP>
+__device__ __forceinline__ int first_particle()
+{
+    return (int)((blockIdx.x % LP) * PT + threadIdx.x) / LP;
+}
+
+// The lanes' sums; every lane of the particle gets the total (a no-op for one lane).
+template <int LP>
+__device__ __forceinline__ float lane_sum(float v)
+{
+    if constexpr (LP > 1) {
+        const unsigned m = ((1u << LP) - 1u) << ((threadIdx.x & 31) & ~(LP - 1));
+#pragma unroll
+        for (int o = 1; o < LP; o <<= 1) v += __shfl_xor_sync(m, v, o);
+    }
+    return v;
+}
+template <int LP>
+__device__ __forceinline__ float2 lane_sum(float2 v)
+{
+    if constexpr (LP == 1) return v;
+    else return f2(lane_sum<LP>(v.x), lane_sum<LP>(v.y));
+}
+template <int LP>
+__device__ __forceinline__ int lane_sum(int v)
+{
+    if constexpr (LP > 1) {
+        const unsigned m = ((1u << LP) - 1u) << ((threadIdx.x & 31) & ~(LP - 1));
+#pragma unroll
+        for (int o = 1; o < LP; o <<= 1) v += __shfl_xor_sync(m, v, o);
+    }
+    return v;
+}
+// Whether this lane writes the particle's results.
+template <int LP>
+__device__ __forceinline__ bool writes()
+{
+    return LP == 1 || (threadIdx.x & (LP - 1)) == 0;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -630,29 +735,27 @@ __device__ __forceinline__ void for_each_candidate(const DevParams &P, const Buf
 
 constexpr int SMEM_AF = HCAP * (16 + 4);
 
+template <int LP>
 __global__ void BOUNDS_A k_pass_a_filter(DevParams P, Bufs b)
 {
-    if (stopped(b) || resorting(b)) return;
+    if (resorting(b)) return;
     __shared__ TileShared ts;
     extern __shared__ __align__(16) unsigned char dsm[];
     float4 *pos = reinterpret_cast<float4 *>(dsm);
     int *sg = reinterpret_cast<int *>(pos + HCAP);
     Tile T;
-    if (!tile_begin(P, b, ts, T)) {
-        if (threadIdx.x == 0) atomicOr(b.err, EB_HALO);
-        return;
-    }
+    if (!tile_begin<LP>(P, b, ts, T)) return;
     for (int t = threadIdx.x; t < T.H; t += PT) {
-        SlotInfo s = slot_info(P, b, ts, T, t);
+        SlotInfo s = slot_info(P, b, ts, t);
         pos[t] = s.e;
         sg[t] = s.g;
     }
     __syncthreads();
-    for (int q = threadIdx.x; q < T.Ni; q += PT) {
-        int si = inner_slot(ts, T, q);
+    for (int q = first_particle<LP>(); q < T.Ni; q += PT) {
+        int si = inner_slot(ts, q);
         int gi = sg[si];
         float4 pi = pos[si];
-        float sw = P.W0;
+        float sw = LP == 1 ? P.W0 : 0.f;
         int c = b.vcnt[gi];
         // one walk over the list words, setting each candidate's neighbour bit by the FP32 test;
         // a candidate inside the rounding band around (3h)^2 (rare) is only noted here and decided
@@ -668,12 +771,14 @@ __global__ void BOUNDS_A k_pass_a_filter(DevParams P, Bufs b)
             nn += (int)in;
             return o | in;
         };
-        uint2 *p = b.vnbr + gi;
-        uint2 nxt = c > 0 ? *p : make_uint2(0u, 0u);   // plain loads: this kernel writes the words
-        int k = 0;
-        for (; k + 3 < c; k += 4, p += P.n) {
+        const int l = threadIdx.x & (LP - 1);   // this lane's words: l, l + LP, ...
+        const size_t stride = (size_t)LP * P.n;
+        uint2 *p = b.vnbr + (size_t)l * P.n + gi;
+        uint2 nxt = 4 * l < c ? *p : make_uint2(0u, 0u);   // plain loads: this kernel writes the words
+        int k = 4 * l;
+        for (; k + 3 < c; k += 4 * LP, p += stride) {
             const uint2 w = nxt;
-            if (k + 4 < c) nxt = p[P.n];   // the next word, in flight while this one is done
+            if (k + 4 * LP < c) nxt = p[stride];   // the next word, in flight while this one is done
             const uint32_t e0 = test(w.x & 0xffffu), e1 = test(w.x >> 16), e2 = test(w.y & 0xffffu),
                            e3 = test(w.y >> 16);
             const uint2 v = make_uint2(e0 | (e1 << 16), e2 | (e3 << 16));
@@ -687,8 +792,8 @@ __global__ void BOUNDS_A k_pass_a_filter(DevParams P, Bufs b)
             if (v.x != w.x || v.y != w.y) *p = v;
         }
         if (band) {   // the band's candidates, decided in FP64 (the FP32 test left their bit 0)
-            uint2 *q = b.vnbr + gi;
-            for (int k0 = 0; k0 < c; k0 += 4, q += P.n) {
+            uint2 *q = b.vnbr + (size_t)l * P.n + gi;
+            for (int k0 = 4 * l; k0 < c; k0 += 4 * LP, q += stride) {
                 uint2 w = *q;
                 uint32_t e[4] = {w.x & 0xffffu, w.x >> 16, w.y & 0xffffu, w.y >> 16};
                 for (int t = 0; t < 4 && k0 + t < c; t++) {
@@ -702,6 +807,9 @@ __global__ void BOUNDS_A k_pass_a_filter(DevParams P, Bufs b)
                 *q = make_uint2(e[0] | (e[1] << 16), e[2] | (e[3] << 16));
             }
         }
+        nn = lane_sum<LP>(nn);
+        if (LP > 1) sw = P.W0 + lane_sum<LP>(sw);
+        if (!writes<LP>()) continue;
         b.nnbr[gi] = nn;
         b.sumW[gi] = sw;
         b.V[gi] = 1.0f / sw;
@@ -716,11 +824,9 @@ __global__ void BOUNDS_A k_pass_a_filter(DevParams P, Bufs b)
 
 constexpr int SMEM_B = HCAP * (16 + 16 + 4 + 4);
 
-template <bool QOLD>
+template <bool QOLD, int LP>
 __global__ void BOUNDS_B k_pass_b(DevParams P, Bufs b)
 {
-    if (stopped(b)) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *b.rebuild = 0u;   // both pass A kernels have run
     __shared__ TileShared ts;
     extern __shared__ __align__(16) unsigned char dsm[];
     float4 *sp = reinterpret_cast<float4 *>(dsm);     // split position
@@ -728,20 +834,18 @@ __global__ void BOUNDS_B k_pass_b(DevParams P, Bufs b)
     float *sv = reinterpret_cast<float *>(sb + HCAP); // V
     int *sg = reinterpret_cast<int *>(sv + HCAP);
     Tile T;
-    if (!tile_begin(P, b, ts, T)) {
-        if (threadIdx.x == 0) atomicOr(b.err, EB_HALO);
-        return;
-    }
+    if (!tile_begin<LP>(P, b, ts, T)) return;
+    if (first_thread()) *b.rebuild = 0u;   // both pass A kernels have run
     for (int t = threadIdx.x; t < T.H; t += PT) {
-        SlotInfo s = slot_info(P, b, ts, T, t);
+        SlotInfo s = slot_info(P, b, ts, t);
         sp[t] = s.e;
         sb[t] = b.mu4[s.g];
         sv[t] = b.V[s.g];
         sg[t] = s.g;
     }
     __syncthreads();
-    for (int q = threadIdx.x; q < T.Ni; q += PT) {
-        int si = inner_slot(ts, T, q);
+    for (int q = first_particle<LP>(); q < T.Ni; q += PT) {
+        int si = inner_slot(ts, q);
         int gi = sg[si];
         float4 pi = sp[si], bi = sb[si];
         // two-lane accumulators: (a11, a12), a22; L rows (l00, l01), (l10, l11); Laplacian sums
@@ -752,7 +856,7 @@ __global__ void BOUNDS_B k_pass_b(DevParams P, Bufs b)
         float a22 = 0.f;
         float di = b.mdr[gi];   // loaded ahead of the neighbour loop
         const float2 ui = f2(bi.x, bi.y), qi = f2(bi.z, bi.w);
-        for_each_candidate<ANN_PF_B>(P, b, gi, [&](int o, int, unsigned) {
+        for_each_candidate<ANN_PF_B, LP>(P, b, gi, [&](int o, int, unsigned) {
             float4 bj = slot_at(sb, o);
             float2 d = pair_d(pi, slot_at(sp, o));
             KernelPowers kp = kernel_powers<true>(len2(d), P);
@@ -775,6 +879,20 @@ __global__ void BOUNDS_B k_pass_b(DevParams P, Bufs b)
                 gq2 = fma2(bc(dq.y), g, gq2);
             }
         });
+        if (LP > 1) {
+            a1 = lane_sum<LP>(a1);
+            a22 = lane_sum<LP>(a22);
+            l0 = lane_sum<LP>(l0);
+            l1 = lane_sum<LP>(l1);
+            rxx = lane_sum<LP>(rxx);
+            rxy = lane_sum<LP>(rxy);
+            ryy = lane_sum<LP>(ryy);
+            if (QOLD) {
+                gq1 = lane_sum<LP>(gq1);
+                gq2 = lane_sum<LP>(gq2);
+            }
+            if (!writes<LP>()) continue;
+        }
         float a11 = a1.x, a12 = a1.y;
         float l00 = l0.x, l01 = l0.y, l10 = l1.x, l11 = l1.y;
         float r1xx = rxx.x, r2xx = rxx.y, r1xy = rxy.x, r2xy = rxy.y, r1yy = ryy.x, r2yy = ryy.y;
@@ -850,10 +968,9 @@ __global__ void BOUNDS_B k_pass_b(DevParams P, Bufs b)
 // the elastic stress tile exists only in the instantiations that read it
 constexpr int smem_c(bool el) { return HCAP * (16 + 16 + (el ? 16 : 0) + 4); }
 
-template <bool QNEW, bool EL>
+template <bool QNEW, bool EL, int LP>
 __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
 {
-    if (stopped(b)) return;
     __shared__ TileShared ts;
     extern __shared__ __align__(16) unsigned char dsm[];
     float4 *sp = reinterpret_cast<float4 *>(dsm);      // split position
@@ -861,13 +978,10 @@ __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
     float4 *se = sb + HCAP;                            // elastic stress (11, 12, 22, -)
     int *sg = reinterpret_cast<int *>(se + (EL ? HCAP : 0));
     Tile T;
-    if (!tile_begin(P, b, ts, T)) {
-        if (threadIdx.x == 0) atomicOr(b.err, EB_HALO);
-        return;
-    }
+    if (!tile_begin<LP>(P, b, ts, T)) return;
     const StateSet out = state_out(b);   // Q^{n+1} (pass B)
     for (int t = threadIdx.x; t < T.H; t += PT) {
-        SlotInfo s = slot_info(P, b, ts, T, t);
+        SlotInfo s = slot_info(P, b, ts, t);
         sp[t] = s.e;
         sb[t] = b.cr[s.g];   // (V, delta_half, Q^{n+1}); pass C reads Q^{n+1} only with QNEW
         if (EL) se[t] = b.pel[s.g];
@@ -878,11 +992,11 @@ __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
     float c0 = fmaxf(10.f * umax, P.c0_min);
     float pref = P.rho0 * c0 * c0 / P.gamma_eos;
     // stability limits of this step's dt (a zero speed gives an infinite limit); pass D then stops
-    if (P.dt_check && blockIdx.x == 0 && threadIdx.x == 0 &&
+    if (P.dt_check && first_thread() &&
         (P.dt > P.dt_static || P.dt * (c0 + umax) * P.inv_h > 0.25f))
         atomicOr(b.err, EB_CFL);
-    for (int q = threadIdx.x; q < T.Ni; q += PT) {
-        int si = inner_slot(ts, T, q);
+    for (int q = first_particle<LP>(); q < T.Ni; q += PT) {
+        int si = inner_slot(ts, q);
         int gi = sg[si];
         float4 pi = sp[si], bi = sb[si];
         float shep = 0.f;
@@ -899,7 +1013,7 @@ __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
         float2 gq1 = f2(0.f, 0.f), gq2 = f2(0.f, 0.f), ge1 = f2(0.f, 0.f), ge2 = f2(0.f, 0.f),
                ge3 = f2(0.f, 0.f);
         const float2 qi = f2(bi.z, bi.w);
-        for_each_candidate<ANN_PF_C>(P, b, gi, [&](int o, int, unsigned) {
+        for_each_candidate<ANN_PF_C, LP>(P, b, gi, [&](int o, int, unsigned) {
             float4 bj = slot_at(sb, o);
             float2 d = pair_d(pi, slot_at(sp, o));
             KernelPowers kp = kernel_powers<true>(len2(d), P);
@@ -920,6 +1034,19 @@ __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
                 }
             }
         });
+        if (LP > 1) {
+            shep = lane_sum<LP>(shep);
+            if (QNEW) {
+                gq1 = lane_sum<LP>(gq1);
+                gq2 = lane_sum<LP>(gq2);
+            }
+            if (EL) {
+                ge1 = lane_sum<LP>(ge1);
+                ge2 = lane_sum<LP>(ge2);
+                ge3 = lane_sum<LP>(ge3);
+            }
+            if (!writes<LP>()) continue;
+        }
         float g1x = gq1.x, g1y = gq1.y, g2x = gq2.x, g2y = gq2.y;
         float e1x = ge1.x, e1y = ge1.y, e2x = ge2.x, e2y = ge2.y, e3x = ge3.x, e3y = ge3.y;
         float dhat = bi.y - P.beta * shep / swi;
@@ -956,10 +1083,9 @@ __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
 // (the (q11, q12)/rho^2 tile exists in the conservative mode only, Pi/rho^2 with the elastic stress)
 constexpr int smem_d(bool cons, bool el) { return HCAP * (16 + 16 + (cons ? 8 : 0) + (cons && el ? 16 : 0) + 4); }
 
-template <bool CONS, bool EL>
+template <bool CONS, bool EL, int LP>
 __global__ void BOUNDS_D k_pass_d(DevParams P, Bufs b)
 {
-    if (stopped(b)) return;
     __shared__ TileShared ts;
     extern __shared__ __align__(16) unsigned char dsm[];
     float4 *sp = reinterpret_cast<float4 *>(dsm);       // split position
@@ -969,15 +1095,12 @@ __global__ void BOUNDS_D k_pass_d(DevParams P, Bufs b)
     int *sg = reinterpret_cast<int *>(se + ((CONS && EL) ? HCAP : 0));
     // the step's output set: Q^{n+1} (pass B) in, the new state out; k_commit of the next step (or
     // the host) commits it if no error has been raised by then
-    if (blockIdx.x == 0 && threadIdx.x == 0) b.ctl[CTL_PENDING] = 1u;
     Tile T;
-    if (!tile_begin(P, b, ts, T)) {
-        if (threadIdx.x == 0) atomicOr(b.err, EB_HALO);
-        return;
-    }
+    if (!tile_begin<LP>(P, b, ts, T)) return;
+    if (first_thread()) b.ctl[CTL_PENDING] = 1u;
     const StateSet out = state_out(b);
     for (int t = threadIdx.x; t < T.H; t += PT) {
-        SlotInfo s = slot_info(P, b, ts, T, t);
+        SlotInfo s = slot_info(P, b, ts, t);
         sp[t] = s.e;
         if (CONS) {
             float rho = P.rho0 * (1.f + reinterpret_cast<const float *>(b.cq + s.g)[2]);
@@ -999,9 +1122,9 @@ __global__ void BOUNDS_D k_pass_d(DevParams P, Bufs b)
         sg[t] = s.g;
     }
     __syncthreads();
-    if (blockIdx.x == 0 && threadIdx.x == 0) *b.maxu = 0u;   // pass C has consumed it
-    for (int q = threadIdx.x; q < T.Ni; q += PT) {
-        int si = inner_slot(ts, T, q);
+    if (first_thread()) *b.maxu = 0u;   // pass C has consumed it
+    for (int q = first_particle<LP>(); q < T.Ni; q += PT) {
+        int si = inner_slot(ts, q);
         int gi = sg[si];
         float4 pi = sp[si], bi = sb[si];
         float2 ci = CONS ? sc[si] : make_float2(0.f, 0.f);
@@ -1021,7 +1144,7 @@ __global__ void BOUNDS_D k_pass_d(DevParams P, Bufs b)
         const float2 ui = f2(bi.z, bi.w);
         float2 w = f2(0.f, 0.f), su = f2(0.f, 0.f), sd = f2(0.f, 0.f);
         float sr = 0.f;
-        for_each_candidate<ANN_PF_D>(P, b, gi, [&](int o, int, unsigned in) {
+        for_each_candidate<ANN_PF_D, LP>(P, b, gi, [&](int o, int, unsigned in) {
             float4 bj = slot_at(sb, o);
             float2 d = pair_d(pi, slot_at(sp, o));
             float r2 = len2(d);
@@ -1057,6 +1180,13 @@ __global__ void BOUNDS_D k_pass_d(DevParams P, Bufs b)
                 sd = fma2(d, bc(rinv2 * kp.rinv), sd);
             }
         });
+        if (LP > 1) {
+            w = lane_sum<LP>(w);
+            su = lane_sum<LP>(su);
+            sd = lane_sum<LP>(sd);
+            sr = lane_sum<LP>(sr);
+            if (!writes<LP>()) continue;
+        }
         const float4 bb = b.bk[gi], cc = b.cq[gi];
         float kri = bb.w, swi = cc.w;
         float B11 = 0.f, B12 = 0.f, B22 = 0.f, dvx = 0.f, dvy = 0.f;
@@ -1200,13 +1330,13 @@ __global__ void __launch_bounds__(PT) k_export_nbrs(DevParams P, Bufs b, int *co
     Tile T;
     if (!tile_begin(P, b, ts, T)) return;
     for (int t = threadIdx.x; t < T.H; t += PT) {
-        SlotInfo s = slot_info(P, b, ts, T, t);
+        SlotInfo s = slot_info(P, b, ts, t);
         pos[t] = s.e;
         sg[t] = s.g;
     }
     __syncthreads();
     for (int q = threadIdx.x; q < T.Ni; q += PT) {
-        int si = inner_slot(ts, T, q);
+        int si = inner_slot(ts, q);
         int gi = sg[si];
         int k = 0;
         for_each_candidate<1>(P, b, gi, [&](int o, int, unsigned in) {
@@ -1241,7 +1371,7 @@ __global__ void __launch_bounds__(PT) k_export_graph(DevParams P, Bufs b, GraphO
     Tile T;
     if (!tile_begin(P, b, ts, T)) return;
     for (int t = threadIdx.x; t < T.H; t += PT) {
-        SlotInfo s = slot_info(P, b, ts, T, t);
+        SlotInfo s = slot_info(P, b, ts, t);
         pos[t] = s.e;
         sg[t] = s.g;
         su[t] = b.mu4[s.g];
@@ -1251,7 +1381,7 @@ __global__ void __launch_bounds__(PT) k_export_graph(DevParams P, Bufs b, GraphO
     __syncthreads();
     const float r2net = 4.f / (P.inv_h * P.inv_h);
     for (int q = threadIdx.x; q < T.Ni; q += PT) {
-        int si = inner_slot(ts, T, q);
+        int si = inner_slot(ts, q);
         int gi = sg[si];
         float4 pi = pos[si], ui = su[si];
         float2 ai = sa[si];
@@ -1330,14 +1460,14 @@ __global__ void __launch_bounds__(PT) k_export_increment(DevParams P, Bufs b, co
     Tile T;
     if (!tile_begin(P, b, ts, T)) return;
     for (int t = threadIdx.x; t < T.H; t += PT) {
-        SlotInfo s = slot_info(P, b, ts, T, t);
+        SlotInfo s = slot_info(P, b, ts, t);
         pos[t] = s.e;
         sg[t] = s.g;
         sa[t] = make_float2(agg1[s.g], agg1[(size_t)P.n + s.g]);
     }
     __syncthreads();
     for (int q = threadIdx.x; q < T.Ni; q += PT) {
-        int si = inner_slot(ts, T, q);
+        int si = inner_slot(ts, q);
         int gi = sg[si];
         float4 pi = pos[si];
         float2 ai = sa[si];
@@ -1437,29 +1567,76 @@ inline int blocks_for(int n, int t) { return (n + t - 1) / t; }
 
 const char *kernel_name(int k) { return (k >= 0 && k < NKERNELS) ? kNames[k] : nullptr; }
 
+namespace {
+
+template <typename F>
+cudaError_t allow_smem(F *f, int bytes)
+{
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
+template <int LP>
+cudaError_t prepare_passes()
+{
+    cudaError_t e;
+    if ((e = allow_smem(k_pass_a_filter<LP>, SMEM_AF))) return e;
+    if ((e = allow_smem(k_pass_b<false, LP>, SMEM_B))) return e;
+    if ((e = allow_smem(k_pass_b<true, LP>, SMEM_B))) return e;
+    if ((e = allow_smem(k_pass_c<false, false, LP>, smem_c(false)))) return e;
+    if ((e = allow_smem(k_pass_c<true, false, LP>, smem_c(false)))) return e;
+    if ((e = allow_smem(k_pass_c<false, true, LP>, smem_c(true)))) return e;
+    if ((e = allow_smem(k_pass_c<true, true, LP>, smem_c(true)))) return e;
+    if ((e = allow_smem(k_pass_d<false, false, LP>, smem_d(false, false)))) return e;
+    if ((e = allow_smem(k_pass_d<true, false, LP>, smem_d(true, false)))) return e;
+    if ((e = allow_smem(k_pass_d<false, true, LP>, smem_d(false, true)))) return e;
+    return allow_smem(k_pass_d<true, true, LP>, smem_d(true, true));
+}
+
+// Pass k (6 to 9) with LP lanes per particle.
+template <int LP>
+void launch_pass(int k, const DevParams &P, const Bufs &b, cudaStream_t s)
+{
+    const dim3 nt(P.tiles * LP, P.tiles);
+    const bool el = P.elastic && !P.conservative;   // the paper momentum takes div Pi from pass C
+    switch (k) {
+    case 6: k_pass_a_filter<LP><<<nt, PT, SMEM_AF, s>>>(P, b); break;
+    case 7:
+        if (P.qnew) k_pass_b<false, LP><<<nt, PT, SMEM_B, s>>>(P, b);
+        else k_pass_b<true, LP><<<nt, PT, SMEM_B, s>>>(P, b);
+        break;
+    case 8:
+        if (P.qnew && el) k_pass_c<true, true, LP><<<nt, PT, smem_c(true), s>>>(P, b);
+        else if (P.qnew) k_pass_c<true, false, LP><<<nt, PT, smem_c(false), s>>>(P, b);
+        else if (el) k_pass_c<false, true, LP><<<nt, PT, smem_c(true), s>>>(P, b);
+        else k_pass_c<false, false, LP><<<nt, PT, smem_c(false), s>>>(P, b);
+        break;
+    case 9:
+        if (P.conservative && P.elastic) k_pass_d<true, true, LP><<<nt, PT, smem_d(true, true), s>>>(P, b);
+        else if (P.conservative) k_pass_d<true, false, LP><<<nt, PT, smem_d(true, false), s>>>(P, b);
+        else if (P.elastic) k_pass_d<false, true, LP><<<nt, PT, smem_d(false, true), s>>>(P, b);
+        else k_pass_d<false, false, LP><<<nt, PT, smem_d(false, false), s>>>(P, b);
+        break;
+    }
+}
+
+}  // namespace
+
 cudaError_t prepare_kernels()
 {
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_pass_a_resort<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_A))) return e;
-    if ((e = cudaFuncSetAttribute(k_pass_a_resort<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_A))) return e;
-    if ((e = cudaFuncSetAttribute(k_pass_a_filter, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_AF))) return e;
-    if ((e = cudaFuncSetAttribute(k_pass_b<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_B))) return e;
-    if ((e = cudaFuncSetAttribute(k_pass_b<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_B))) return e;
-    if ((e = cudaFuncSetAttribute(k_pass_c<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_c(false)))) return e;
-    if ((e = cudaFuncSetAttribute(k_pass_c<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_c(false)))) return e;
-    if ((e = cudaFuncSetAttribute(k_pass_c<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_c(true)))) return e;
-    if ((e = cudaFuncSetAttribute(k_pass_c<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_c(true)))) return e;
-    if ((e = cudaFuncSetAttribute(k_pass_d<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_d(false, false)))) return e;
-    if ((e = cudaFuncSetAttribute(k_pass_d<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_d(true, false)))) return e;
-    if ((e = cudaFuncSetAttribute(k_pass_d<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_d(false, true)))) return e;
-    if ((e = cudaFuncSetAttribute(k_pass_d<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_d(true, true)))) return e;
-    return cudaSuccess;
+    if ((e = allow_smem(k_pass_a_resort<false>, SMEM_A))) return e;
+    if ((e = allow_smem(k_pass_a_resort<true>, SMEM_A))) return e;
+    if ((e = prepare_passes<1>())) return e;
+    if ((e = prepare_passes<2>())) return e;
+    if ((e = prepare_passes<4>())) return e;
+    return prepare_passes<8>();
 }
 
 // Kernel k of the step on stream s (see kNames).
 cudaError_t launch_kernel(int k, const DevParams &P, const Bufs &b, cudaStream_t s)
 {
-    int nb = blocks_for(P.n, 256), nt = P.tiles * P.tiles;
+    const int nb = blocks_for(P.n, 256);
+    const dim3 nt(P.tiles, P.tiles);
     switch (k) {
     case 0: k_predict<<<nb, 256, 0, s>>>(P, b); break;
     case 1: k_keys<<<nb, 256, 0, s>>>(P, b); break;
@@ -1467,24 +1644,11 @@ cudaError_t launch_kernel(int k, const DevParams &P, const Bufs &b, cudaStream_t
     case 3: k_scatter<<<nb, 256, 0, s>>>(P, b); break;
     case 4: k_cell_order<<<blocks_for(P.ncell, 8), 256, 0, s>>>(P, b); break;
     case 5: k_pass_a_resort<false><<<nt, PT, SMEM_A, s>>>(P, b); break;
-    case 6: k_pass_a_filter<<<nt, PT, SMEM_AF, s>>>(P, b); break;
-    case 7:
-        if (P.qnew) k_pass_b<false><<<nt, PT, SMEM_B, s>>>(P, b);
-        else k_pass_b<true><<<nt, PT, SMEM_B, s>>>(P, b);
-        break;
-    case 8: {
-        bool el = P.elastic && !P.conservative;   // the paper momentum takes div Pi from here
-        if (P.qnew && el) k_pass_c<true, true><<<nt, PT, smem_c(true), s>>>(P, b);
-        else if (P.qnew) k_pass_c<true, false><<<nt, PT, smem_c(false), s>>>(P, b);
-        else if (el) k_pass_c<false, true><<<nt, PT, smem_c(true), s>>>(P, b);
-        else k_pass_c<false, false><<<nt, PT, smem_c(false), s>>>(P, b);
-        break;
-    }
-    case 9:
-        if (P.conservative && P.elastic) k_pass_d<true, true><<<nt, PT, smem_d(true, true), s>>>(P, b);
-        else if (P.conservative) k_pass_d<true, false><<<nt, PT, smem_d(true, false), s>>>(P, b);
-        else if (P.elastic) k_pass_d<false, true><<<nt, PT, smem_d(false, true), s>>>(P, b);
-        else k_pass_d<false, false><<<nt, PT, smem_d(false, false), s>>>(P, b);
+    case 6: case 7: case 8: case 9:
+        if (P.lanes == 8) launch_pass<8>(k, P, b, s);
+        else if (P.lanes == 4) launch_pass<4>(k, P, b, s);
+        else if (P.lanes == 2) launch_pass<2>(k, P, b, s);
+        else launch_pass<1>(k, P, b, s);
         break;
     default: return cudaErrorInvalidValue;
     }
@@ -1520,7 +1684,7 @@ cudaError_t enqueue_search(const DevParams &P, const Bufs &b, cudaStream_t s)
 
 cudaError_t enqueue_candidates_from_ref(const DevParams &P, const Bufs &b, cudaStream_t s)
 {
-    k_pass_a_resort<true><<<P.tiles * P.tiles, PT, SMEM_A, s>>>(P, b);
+    k_pass_a_resort<true><<<dim3(P.tiles, P.tiles), PT, SMEM_A, s>>>(P, b);
     return cudaGetLastError();
 }
 
@@ -1548,14 +1712,14 @@ cudaError_t enqueue_export_graph(const DevParams &P, const Bufs &b, const GraphO
     cudaError_t e = cudaFuncSetAttribute(k_export_graph, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_EX);
     if (!e) e = cudaFuncSetAttribute(k_export_increment, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_EX);
     if (e) return e;
-    k_export_graph<<<P.tiles * P.tiles, PT, SMEM_EX, s>>>(P, b, o);
-    k_export_increment<<<P.tiles * P.tiles, PT, HCAP * (16 + 8 + 4), s>>>(P, b, o.agg1, o.tend_id, kdt, inc);
+    k_export_graph<<<dim3(P.tiles, P.tiles), PT, SMEM_EX, s>>>(P, b, o);
+    k_export_increment<<<dim3(P.tiles, P.tiles), PT, HCAP * (16 + 8 + 4), s>>>(P, b, o.agg1, o.tend_id, kdt, inc);
     return cudaGetLastError();
 }
 
 cudaError_t enqueue_export_nbrs(const DevParams &P, const Bufs &b, int *cols_tmp, cudaStream_t s)
 {
-    k_export_nbrs<<<P.tiles * P.tiles, PT, SMEM_AF, s>>>(P, b, cols_tmp);
+    k_export_nbrs<<<dim3(P.tiles, P.tiles), PT, SMEM_AF, s>>>(P, b, cols_tmp);
     return cudaGetLastError();
 }
 
