@@ -459,6 +459,10 @@ int ann_surrogate_set_scales(ann_surrogate *sg, double us, double ys_q, double y
  * (~21 on a lattice); a denser cluster returns NBR_OVERFLOW instead of dropping neighbours. */
 int ann_surrogate_load(ann_surrogate *sg, ann_ctx *ctx, const float *tend);
 
+/* ann_surrogate_load with host tendencies particle by particle (n x 8 FP32: component c of particle ID i
+ * at 8 i + c; not NULL): the device sorts them into components. */
+int ann_surrogate_load_rows(ann_surrogate *sg, ann_ctx *ctx, const float *tend);
+
 /* Network outputs y of the loaded state: host n x 4 FP32, ID order (may be NULL). */
 int ann_surrogate_forward(ann_surrogate *sg, float *y);
 

@@ -148,6 +148,7 @@ def lib() -> ctypes.CDLL:
         "ann_surrogate_get_params": (i32, [vp, _P(ctypes.c_float)]),
         "ann_surrogate_set_scales": (i32, [vp, ctypes.c_double, ctypes.c_double, ctypes.c_double, i32]),
         "ann_surrogate_load": (i32, [vp, vp, _P(ctypes.c_float)]),
+        "ann_surrogate_load_rows": (i32, [vp, vp, _P(ctypes.c_float)]),
         "ann_surrogate_forward": (i32, [vp, _P(ctypes.c_float)]),
         "ann_surrogate_euler": (i32, [vp, _P(ctypes.c_float)]),
         "ann_surrogate_gradients": (i32, [vp, _P(ctypes.c_float), _P(ctypes.c_double), _P(ctypes.c_float)]),
@@ -705,6 +706,10 @@ def _tend(tend):
 
 def ann_surrogate_load(sg, ctx, tend=None) -> None:
     """tend: None (the context's last recorded step) or (n, 8) tendencies in ID order."""
+    if tend is not None and np.ndim(tend) == 2 and np.shape(tend)[1] == 8:   # the device sorts the rows
+        rows = np.ascontiguousarray(tend, dtype=np.float32)
+        _scheck(lib().ann_surrogate_load_rows(sg, ctx, _fp(rows)), sg, "ann_surrogate_load")
+        return
     ptr, keep = _tend(tend)
     _scheck(lib().ann_surrogate_load(sg, ctx, ptr), sg, "ann_surrogate_load")
 

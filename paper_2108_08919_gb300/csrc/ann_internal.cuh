@@ -258,6 +258,28 @@ cudaError_t enqueue_gemm_tn(const void *A, int K, const void *B, int N, int rows
 cudaError_t enqueue_layer(const void *A1, int K1, const void *A2, int K2, const void *W, const float *bw,
                           const void *P, const float *bp, int Np, void *H, void *Z, int z_bf16, int rows,
                           unsigned *err, int max_ctas, cudaStream_t s);
+// One layer backward: dA = ([A1 W1^T] + [A2 W2^T]) masked by Hin > 0 (BF16, rows x 128), Z = dA P^T (FP32,
+// rows x Np).  W1 128 x K1, W2 128 x K2, P Np x 128, BF16, 16-byte aligned.
+cudaError_t enqueue_layer_bwd(const void *A1, int K1, const void *W1, const void *A2, int K2, const void *W2,
+                              const void *Hin, const void *P, int Np, void *dA, float *Z, int rows, unsigned *err,
+                              cudaStream_t s);
+// Weight gradients: part (wgrad_ctas(rows) x 128 x (n1 + n2 + 16 if bias)) = A^T [B1 | B2 | 1] per CTA, A rows x 128,
+// B1 and B2 rows x n1, n2 (BF16); enqueue_wgrad_sum adds the CTAs' parts of several products.
+constexpr int WGRAD_CTAS = 152;
+int wgrad_ctas(int rows);
+cudaError_t enqueue_wgrad(const void *A, const void *B1, int n1, const void *B2, int n2, bool bias, int rows, float *part,
+                          unsigned *err, cudaStream_t s);
+struct WgradOut {
+    struct Product {
+        const float *part;
+        int n, n1, n2;      // n = n1 + n2, + 16 with a bias
+        int transposed;     // 0: w is 128 x (n1 + n2); 1: w is keep x 128 (columns are w's rows)
+        int keep;
+        float *w, *b;       // gradients of the weight and of the bias (column n1 + n2)
+    } p[6];
+    int count, ctas;
+};
+cudaError_t enqueue_wgrad_sum(const WgradOut &o, cudaStream_t s);
 cudaError_t enqueue_unwrapped(const DevParams &P, const Bufs &b, int *inv, const long long *ids, int k, double *xy,
                               cudaStream_t s);
 

@@ -1,7 +1,10 @@
 // BF16 tensor-core GEMMs for the learned surrogate (5th-generation tensor cores, tcgen05, sm_103a):
 //
 //   nt:  C[rows x N] = act([A1 | A2][rows x (K1 + K2)] . B[N x K]^T + bias)   (forward, dX)
-//   tn:  C[K x N]   += A[rows x K]^T . B[rows x N]                              (weight gradients)
+//   tn:  C[K x N]   += A[rows x K]^T . B[rows x N]                              (row reductions)
+//
+// (the stand-alone entry points; the surrogate's layers, forward and backward, and its weight gradients have
+// kernels of their own below).
 //
 // A, B are BF16, accumulation FP32 in tensor memory.  One CTA of 128 threads: thread 0 issues
 // tcgen05.mma (M = 128, K = 16 per instruction) from shared-memory descriptors, the completion is
@@ -53,6 +56,21 @@ __device__ __forceinline__ uint64_t smem_desc_sw(uint32_t addr, uint32_t span)
     return d;
 }
 
+// Descriptor of an M/N-major operand in the same box: rows of the box are the K index, `span` bytes of
+// a row are M/N, K groups of 8 rows are 8 span bytes apart (SBO), and the next span / 2 columns follow in
+// the next box, `box` bytes on (LBO).
+__device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr, uint32_t span, uint32_t box)
+{
+    const uint64_t mode = span == 128 ? 2u : (span == 64 ? 4u : 6u);
+    uint64_t d = 0;
+    d |= (uint64_t)((addr >> 4) & 0x3FFFu);
+    d |= (uint64_t)((box >> 4) & 0x3FFFu) << 16;
+    d |= (uint64_t)(((8u * span) >> 4) & 0x3FFFu) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= mode << 61;
+    return d;
+}
+
 // Byte offset of 16-byte chunk j of row r in a swizzled box with rows of `span` bytes.
 __device__ __forceinline__ uint32_t sw_off(int r, int j, uint32_t span)
 {
@@ -60,10 +78,12 @@ __device__ __forceinline__ uint32_t sw_off(int r, int j, uint32_t span)
     return (uint32_t)r * span + ((uint32_t)(j ^ x) << 4);
 }
 
-// Instruction descriptor of kind::f16: D FP32, A and B BF16, both K-major, N >> 3, M >> 4.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N)
+// Instruction descriptor of kind::f16: D FP32, A and B BF16, each K-major or (a_mn, b_mn) M/N-major,
+// N >> 3, M >> 4.
+__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool a_mn = false, bool b_mn = false)
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) |
+           ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void tmem_alloc(uint32_t *holder, uint32_t ncols)
@@ -320,8 +340,10 @@ struct LayerMaps {
 };
 
 struct LayerArgs {
-    const __nv_bfloat16 *W;   // 128 x K
-    const float *bw;          // 128
+    const __nv_bfloat16 *W;   // 128 x K; backward: 128 x K1
+    const __nv_bfloat16 *W2;  // backward: 128 x K2
+    const __nv_bfloat16 *Hin; // backward: rows x 128, the layer's activations
+    const float *bw;          // 128 (forward)
     const __nv_bfloat16 *P;   // Np x 128
     const float *bp;          // Np or null
     int rows, K1, K2, Np, z_bf16, store_h, stages;
@@ -391,6 +413,14 @@ __device__ __forceinline__ void layer_load(const LayerMaps &m, int K1, int K2, i
     for (int c = 0; c < K2; c += (int)s2 / 2, d += MT * s2) tma_load_2d(d, &m.a2, c, r0, mb);
 }
 
+// BWD: one layer of the backward pass with the same machinery,
+//   da = ([A1 W1^T] + [A2 W2^T]) where the layer's activation is positive, 0 elsewhere (relu)
+//   z  = da . P^T                                                          (FP32)
+// The two products have accumulators of their own (h's and z's columns: z is issued after both are
+// read) and are added in FP32, as if each had been stored; da goes to H in BF16.  The 65,536-row training step spent
+// 33 us on each product through an unpipelined kernel, 38 us on each relu mask and 38 us on each bias
+// gradient's column sums as kernels of their own; a fused layer takes 17 to 21 us.
+template <bool BWD>
 __global__ void __launch_bounds__(LT, 1) k_layer(const __grid_constant__ LayerMaps maps, LayerArgs a)
 {
     extern __shared__ __align__(128) unsigned char sm_raw[];
@@ -426,14 +456,16 @@ __global__ void __launch_bounds__(LT, 1) k_layer(const __grid_constant__ LayerMa
     }
     for (int e = tid; e < HW * (K / 8); e += LT) {
         int r = e / (K / 8), k8 = (e % (K / 8)) * 8;
-        *reinterpret_cast<uint4 *>(sW + kmaj_off(r, k8, K)) = *reinterpret_cast<const uint4 *>(a.W + (size_t)r * K + k8);
+        const __nv_bfloat16 *src = !BWD ? a.W + (size_t)r * K + k8
+                                   : (k8 < a.K1 ? a.W + (size_t)r * a.K1 + k8 : a.W2 + (size_t)r * a.K2 + (k8 - a.K1));
+        *reinterpret_cast<uint4 *>(sW + kmaj_off(r, k8, K)) = *reinterpret_cast<const uint4 *>(src);
     }
     for (int e = tid; e < Np * (HW / 8); e += LT) {
         int r = e / (HW / 8), k8 = (e % (HW / 8)) * 8;
         *reinterpret_cast<uint4 *>(sP + kmaj_off(r, k8, HW)) = *reinterpret_cast<const uint4 *>(a.P + (size_t)r * HW + k8);
     }
     if (tid < HW) {
-        sbw[tid] = a.bw[tid];
+        sbw[tid] = BWD ? 0.f : a.bw[tid];
         sbp[tid] = (a.bp && tid < Np) ? a.bp[tid] : 0.f;
     }
     fence_async_smem();
@@ -468,8 +500,10 @@ __global__ void __launch_bounds__(LT, 1) k_layer(const __grid_constant__ LayerMa
                         const uint32_t span = part_span(C);
                         for (int c = 0; c < C; c += 16, kk += 16) {
                             const uint32_t in_box = (uint32_t)(c % ((int)span / 2)) * 2;
-                            mma_bf16(tmem + (uint32_t)b * 256u, smem_desc_sw(box + in_box, span),
-                                     smem_desc(smem_u32(sW) + (uint32_t)(kk / 8) * 128, 128, sbo_w), idesc1, kk > 0);
+                            mma_bf16(tmem + (uint32_t)b * 256u + (BWD && part ? (uint32_t)HW : 0u),
+                                     smem_desc_sw(box + in_box, span),
+                                     smem_desc(smem_u32(sW) + (uint32_t)(kk / 8) * 128, 128, sbo_w), idesc1,
+                                     BWD ? c > 0 : kk > 0);
                             if (in_box + 32 == span) box += MT * span;
                         }
                     }
@@ -515,22 +549,49 @@ __global__ void __launch_bounds__(LT, 1) k_layer(const __grid_constant__ LayerMa
             // stores commit two groups a tile, h then z: once at most the last (z of tile i - 1) is
             // still reading, sH (stored from by tile i - 1) and sZ of buffer b (by tile i - 2) are free
             if (leader && i >= 1) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+            uint4 act[8];   // backward: this thread's 64 activations, in flight while the products run
+            if (BWD) {
+                const int gr = t * MT + row;
+                const uint4 *src = reinterpret_cast<const uint4 *>(a.Hin + (size_t)gr * HW + half * (HW / 2));
+#pragma unroll
+                for (int q = 0; q < 8; q++) act[q] = gr < a.rows ? __ldg(src + q) : make_uint4(0u, 0u, 0u, 0u);
+            }
             ok = epi_all(mbar_wait(&acc1_full[b], (uint32_t)(i / 2) & 1u));
             if (!ok) break;
             fence_after();
             // h: bias, relu, BF16 into sH; 64 columns per warp, 32 at a time
-            for (int c0 = half * (HW / 2); c0 < (half + 1) * (HW / 2); c0 += 32) {
+#pragma unroll
+            for (int cc = 0; cc < HW / 2; cc += 32) {
+                const int c0 = half * (HW / 2) + cc;
                 uint32_t r[32];
                 tmem_ld16_async(acc + (uint32_t)c0, r);
                 tmem_ld16_async(acc + (uint32_t)(c0 + 16), r + 16);
                 tmem_ld_wait();
                 uint4 w[4];
                 __nv_bfloat162 *h2 = reinterpret_cast<__nv_bfloat162 *>(w);
+                if (BWD) {
+                    if (a.K2 > 0) {
+                        uint32_t r2[32];
+                        tmem_ld16_async(acc + (uint32_t)(HW + c0), r2);
+                        tmem_ld16_async(acc + (uint32_t)(HW + c0 + 16), r2 + 16);
+                        tmem_ld_wait();
 #pragma unroll
-                for (int k = 0; k < 16; k++) {
-                    const float2 bb = *reinterpret_cast<const float2 *>(sbw + c0 + 2 * k);
-                    h2[k] = __floats2bfloat162_rn(fmaxf(__uint_as_float(r[2 * k]) + bb.x, 0.f),
-                                                  fmaxf(__uint_as_float(r[2 * k + 1]) + bb.y, 0.f));
+                        for (int k = 0; k < 32; k++) r[k] = __float_as_uint(__uint_as_float(r2[k]) + __uint_as_float(r[k]));
+                    }
+                    const __nv_bfloat162 *av = reinterpret_cast<const __nv_bfloat162 *>(act + cc / 8);
+#pragma unroll
+                    for (int k = 0; k < 16; k++) {
+                        const float2 hv = __bfloat1622float2(av[k]);
+                        h2[k] = __floats2bfloat162_rn(hv.x > 0.f ? __uint_as_float(r[2 * k]) : 0.f,
+                                                      hv.y > 0.f ? __uint_as_float(r[2 * k + 1]) : 0.f);
+                    }
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 16; k++) {
+                        const float2 bb = *reinterpret_cast<const float2 *>(sbw + c0 + 2 * k);
+                        h2[k] = __floats2bfloat162_rn(fmaxf(__uint_as_float(r[2 * k]) + bb.x, 0.f),
+                                                      fmaxf(__uint_as_float(r[2 * k + 1]) + bb.y, 0.f));
+                    }
                 }
 #pragma unroll
                 for (int q = 0; q < 4; q++) {   // chunk j of the 64-column box c0 / 64
@@ -539,6 +600,7 @@ __global__ void __launch_bounds__(LT, 1) k_layer(const __grid_constant__ LayerMa
                 }
             }
             fence_async_smem();
+            if (BWD) fence_before();   // the product z overwrites the columns read above
             mbar_arrive(&h_full[b]);
             epi_sync();
             if (leader) {
@@ -592,7 +654,7 @@ __global__ void __launch_bounds__(LT, 1) k_layer(const __grid_constant__ LayerMa
 }
 
 // ------------------------------------------------------------------------------------------------
-// tn: C[K x N] += A^T B over all rows.  CTA (x, y): feature block y (128 features of A's K), row
+// tn (the stand-alone entry point): C[K x N] += A^T B over all rows.  CTA (x, y): feature block y (128 features of A's K), row
 // chunks x, x + gridDim.x, ...; the chunk of 128 rows is staged transposed (features x rows and
 // N x rows, both K-major in the rows) and reduced by 8 MMAs of K = 16 rows into TMEM; at the end
 // the CTA adds its 128 x N partial to C with FP32 atomics.
@@ -706,6 +768,157 @@ __global__ void __launch_bounds__(128) k_gemm_tn(TnArgs a)
     if (warp == 0) tmem_dealloc(tmem, ncols);
 }
 
+// ------------------------------------------------------------------------------------------------
+// wgrad: the weight gradients of training,  part[cta] = A^T [B1 | B2 | 1]  over the CTA's row tiles,
+// 128 x (n1 + n2 + 16) FP32 in tensor memory.  A (rows x 128) and B (rows x n) are the row-major
+// activations and adjoints as stored: TMA lands 128-row boxes, whose rows are the K index, so both
+// operands are M/N-major and nothing is transposed (k_gemm_tn below transposes through registers with
+// two-byte shared stores: 27 to 50 us a product at 65,536 rows, 418 us a training step).  The block of
+// ones gives the column sums of A, the bias gradient, in its first column.  Warp 4's first lane loads
+// and issues; warps 0-3 write the CTA's partial sums, which k_wgrad_sum adds in CTA order (so the
+// gradients are reproducible).  8 to 15 us a product.
+// ------------------------------------------------------------------------------------------------
+
+struct WgradMaps {
+    CUtensorMap a, b1, b2;
+};
+
+struct WgradArgs {
+    int rows, n1, n2, bias;   // widths of B1, B2 (0: none) and 16 for the column sums or 0
+    float *part;              // gridDim.x x 128 x (n1 + n2 + bias)
+    unsigned *err;
+};
+
+constexpr int WG_STAGES = 2;
+constexpr int WG_THREADS = 160;
+
+__global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad(const __grid_constant__ WgradMaps maps, WgradArgs a)
+{
+    extern __shared__ __align__(128) unsigned char sm_raw[];
+    __shared__ uint64_t full[WG_STAGES], empty[WG_STAGES], done;
+    __shared__ uint32_t tbase;
+    unsigned char *sm = sm_raw + ((1024u - (smem_u32(sm_raw) & 1023u)) & 1023u);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int n = a.n1 + a.n2 + a.bias;
+    const uint32_t s1 = part_span(a.n1), s2 = part_span(a.n2);
+    const uint32_t abytes = MT * HW * 2, b1bytes = (uint32_t)MT * a.n1 * 2, b2bytes = (uint32_t)MT * a.n2 * 2;
+    const uint32_t stage = abytes + b1bytes + b2bytes;   // multiples of 1024 bytes each
+    unsigned char *ones = sm + (size_t)WG_STAGES * stage;   // 16 x 128 BF16
+    const int ntiles = (a.rows + MT - 1) / MT;
+    const int mine = (int)blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    if (warp == 0) tmem_alloc(&tbase, 256);
+    if (tid == 0) {
+        for (int q = 0; q < WG_STAGES; q++) {
+            mbar_init(&full[q], 1);
+            mbar_init(&empty[q], 1);
+        }
+        mbar_init(&done, 1);
+    }
+    for (int e = tid; e < 16 * MT / 2; e += WG_THREADS) reinterpret_cast<uint32_t *>(ones)[e] = 0x3f803f80u;   // 1.0, 1.0
+    fence_async_smem();
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = tbase;
+    if (warp == 4) {
+        if (lane == 0) {
+            const uint32_t id1 = idesc_bf16(MT, a.n1, true, true), id2 = idesc_bf16(MT, a.n2 > 0 ? a.n2 : 16, true, true),
+                           id3 = idesc_bf16(MT, 16, true, false);
+            auto load = [&](int i) {
+                const int q = i % WG_STAGES, r0 = ((int)blockIdx.x + i * (int)gridDim.x) * MT;
+                const uint32_t mb = smem_u32(&full[q]);
+                uint32_t d = smem_u32(sm) + (uint32_t)q * stage;
+                mbar_expect(&full[q], stage);
+                for (int c = 0; c < HW; c += 64, d += MT * 128) tma_load_2d(d, &maps.a, c, r0, mb);
+                for (int c = 0; c < a.n1; c += (int)s1 / 2, d += MT * s1) tma_load_2d(d, &maps.b1, c, r0, mb);
+                for (int c = 0; c < a.n2; c += (int)s2 / 2, d += MT * s2) tma_load_2d(d, &maps.b2, c, r0, mb);
+            };
+            bool ok = true;
+            int issued = 0, consumed = 0;
+            for (; issued < WG_STAGES && issued < mine; issued++) load(issued);
+            for (int i = 0; i < mine; i++) {
+                const int q = i % WG_STAGES;
+                ok = mbar_wait(&full[q], (uint32_t)(i / WG_STAGES) & 1u);
+                if (!ok) break;
+                consumed++;
+                fence_after();
+                const uint32_t sa = smem_u32(sm) + (uint32_t)q * stage, sb1 = sa + abytes, sb2 = sb1 + b1bytes;
+                for (int k = 0; k < MT / 16; k++) {   // 16 rows of the box a step
+                    const uint64_t da = smem_desc_mn(sa + (uint32_t)k * 16 * 128, 128, MT * 128);
+                    mma_bf16(tmem, da, smem_desc_mn(sb1 + (uint32_t)k * 16 * s1, s1, MT * s1), id1, i > 0 || k > 0);
+                    if (a.n2 > 0)
+                        mma_bf16(tmem + (uint32_t)a.n1, da, smem_desc_mn(sb2 + (uint32_t)k * 16 * s2, s2, MT * s2), id2,
+                                 i > 0 || k > 0);
+                    if (a.bias > 0)
+                        mma_bf16(tmem + (uint32_t)(a.n1 + a.n2), da, smem_desc(smem_u32(ones), 128, 256), id3,
+                                 i > 0 || k > 0);
+                }
+                mma_commit(&empty[q]);
+                if (issued < mine) {
+                    ok = mbar_wait(&empty[q], (uint32_t)(i / WG_STAGES) & 1u);
+                    if (!ok) break;
+                    load(issued++);
+                }
+            }
+            if (ok) mma_commit(&done);
+            else atomicOr(a.err, 8u);
+            // loads issued for tiles that were not reached (only after a failed wait) land before exit
+            for (int i = consumed; i < issued; i++) mbar_wait(&full[i % WG_STAGES], (uint32_t)(i / WG_STAGES) & 1u);
+        }
+        __syncwarp();
+    } else if (mine > 0) {
+        const bool ok = mbar_wait(&done, 0u);
+        if (__all_sync(0xffffffffu, ok)) {
+            fence_after();
+            const int m = warp * 32 + lane;   // feature of A
+            float *dst = a.part + ((size_t)blockIdx.x * MT + m) * n;
+            for (int c0 = 0; c0 < n; c0 += 16) {
+                float v[16];
+                tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+#pragma unroll
+                for (int k = 0; k < 4; k++)
+                    reinterpret_cast<float4 *>(dst + c0)[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+            }
+        } else if (lane == 0) {
+            atomicOr(a.err, 8u);
+        }
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    if (warp == 0) tmem_dealloc(tmem, 256);
+}
+
+// Sums the CTAs' partials of several products and writes the gradients: element (m, c) of product p goes to
+// its weight's place (see WgradOut).  A block takes 32 elements, 8 threads each (every eighth CTA), and
+// joins them in a fixed order; 37 MB of partials (one thread per element: 47 us of latency).
+__global__ void __launch_bounds__(256) k_wgrad_sum(WgradOut o)
+{
+    __shared__ float red[8][32];
+    const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
+    int e = blockIdx.x * 32 + lane, p = 0;   // 128 n elements a product: a block has one product
+    while (p < o.count && e >= MT * o.p[p].n) e -= MT * o.p[p++].n;
+    if (p == o.count) return;
+    const WgradOut::Product &q = o.p[p];
+    const float *src = q.part + e;   // (m, c) at m n + c
+    const size_t stride = (size_t)MT * q.n;
+    float s = 0.f;
+#pragma unroll 5
+    for (int g = slice; g < o.ctas; g += 8) s += __ldg(src + (size_t)g * stride);
+    red[slice][lane] = s;
+    __syncthreads();
+    if (slice) return;
+    s = ((red[0][lane] + red[1][lane]) + (red[2][lane] + red[3][lane])) +
+        ((red[4][lane] + red[5][lane]) + (red[6][lane] + red[7][lane]));
+    const int m = e / q.n, c = e % q.n;
+    if (c < q.n1 + q.n2) {
+        if (!q.transposed) q.w[(size_t)m * (q.n1 + q.n2) + c] = s;
+        else if (c < q.keep) q.w[(size_t)c * MT + m] = s;
+    } else if (c == q.n1 + q.n2) {
+        q.b[m] = s;
+    }
+}
+
 // Self-test of the bounded wait: one thread polls an mbarrier that nothing completes (a fresh
 // barrier's phase 0 never finishes) and, after `limit` polls, raises the flag exactly as an
 // expired wait of the tensor-core kernels does.
@@ -785,11 +998,21 @@ bool part_ok(int C, int es = 2) { return C * es == 32 || C * es == 64 || (C * es
 
 }  // namespace
 
-cudaError_t enqueue_layer(const void *A1, int K1, const void *A2, int K2, const void *W, const float *bw,
-                          const void *P, const float *bp, int Np, void *H, void *Z, int z_bf16, int rows,
-                          unsigned *err, int max_ctas, cudaStream_t s)
+namespace {
+
+cudaError_t sm_count(int *sms)
 {
-    const int K = K1 + K2;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    return e ? e : cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+}
+
+// Maps, shared memory and launch of a layer kernel.
+template <bool BWD>
+cudaError_t launch_layer(const void *A1, const void *A2, void *H, void *Z, LayerArgs a, int max_ctas, cudaStream_t s)
+{
+    const int K1 = a.K1, K2 = a.K2, K = K1 + K2, Np = a.Np, rows = a.rows;
+    const bool z_bf16 = a.z_bf16 != 0;
     if (K < 16 || K > 256 || K % 16 || K1 % 16 || K1 < 16 || Np < 16 || Np > 128 || Np % 16 || rows < 0 ||
         (K2 > 0 && !A2) || !part_ok(K1) || (K2 > 0 && !part_ok(K2)) || !part_ok(Np, z_bf16 ? 2 : 4) ||
         (z_bf16 ? 2 : 4) * Np > 128)
@@ -800,8 +1023,6 @@ cudaError_t enqueue_layer(const void *A1, int K1, const void *A2, int K2, const 
     if (!row_map(&maps.a1, A1, rows, K1, false) || (K2 > 0 && !row_map(&maps.a2, A2, rows, K2, false)) ||
         (H && !row_map(&maps.h, H, rows, HW, false)) || !row_map(&maps.z, Z, rows, Np, !z_bf16))
         return cudaErrorInvalidValue;
-    LayerArgs a{static_cast<const __nv_bfloat16 *>(W), bw, static_cast<const __nv_bfloat16 *>(P), bp,
-                rows, K1, K2, Np, z_bf16, H ? 1 : 0, 2, err};
     // W, P, an h tile, two z tiles and a ring of 2 to 4 A tiles in at most 216 KB; at least 116 KB,
     // so that one CTA (all 512 TMEM columns) runs per SM
     const size_t zbytes = (size_t)MT * Np * (z_bf16 ? 2 : 4);
@@ -813,19 +1034,68 @@ cudaError_t enqueue_layer(const void *A1, int K1, const void *A2, int K2, const 
     if (a.stages < 2) a.stages = 2;
     size_t smem = fixed + (size_t)a.stages * abytes + 1024;   // + alignment slack
     if (smem < 116 * 1024) smem = 116 * 1024;
-    cudaError_t e = cudaFuncSetAttribute(k_layer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_layer<BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int sms = 0;
+    if (!e) e = sm_count(&sms);
     if (e) return e;
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        e = cudaGetDevice(&dev);
-        if (!e) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e) return e;
-    }
     int tiles = (rows + MT - 1) / MT;
     int g = tiles < sms ? tiles : sms;
     if (max_ctas > 0 && g > max_ctas) g = max_ctas;
-    k_layer<<<g, LT, smem, s>>>(maps, a);
+    k_layer<BWD><<<g, LT, smem, s>>>(maps, a);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t enqueue_layer(const void *A1, int K1, const void *A2, int K2, const void *W, const float *bw,
+                          const void *P, const float *bp, int Np, void *H, void *Z, int z_bf16, int rows,
+                          unsigned *err, int max_ctas, cudaStream_t s)
+{
+    LayerArgs a{static_cast<const __nv_bfloat16 *>(W), nullptr, nullptr, bw, static_cast<const __nv_bfloat16 *>(P), bp,
+                rows, K1, K2, Np, z_bf16, H ? 1 : 0, 2, err};
+    return launch_layer<false>(A1, A2, H, Z, a, max_ctas, s);
+}
+
+cudaError_t enqueue_layer_bwd(const void *A1, int K1, const void *W1, const void *A2, int K2, const void *W2,
+                              const void *Hin, const void *P, int Np, void *dA, float *Z, int rows, unsigned *err,
+                              cudaStream_t s)
+{
+    LayerArgs a{static_cast<const __nv_bfloat16 *>(W1), static_cast<const __nv_bfloat16 *>(W2),
+                static_cast<const __nv_bfloat16 *>(Hin), nullptr, static_cast<const __nv_bfloat16 *>(P), nullptr,
+                rows, K1, K2, Np, 0, 1, 2, err};
+    return launch_layer<true>(A1, A2, dA, Z, a, 0, s);
+}
+
+int wgrad_ctas(int rows)
+{
+    const int tiles = (rows + MT - 1) / MT;
+    return tiles < WGRAD_CTAS ? tiles : WGRAD_CTAS;
+}
+
+cudaError_t enqueue_wgrad(const void *A, const void *B1, int n1, const void *B2, int n2, bool bias, int rows, float *part,
+                          unsigned *err, cudaStream_t s)
+{
+    if (rows < 1 || n1 < 16 || n1 > 128 || !part_ok(n1) || n2 < 0 || n2 > 64 || (n2 > 0 && !part_ok(n2)))
+        return cudaErrorInvalidValue;
+    WgradMaps maps;
+    std::memset(&maps, 0, sizeof maps);
+    if (!row_map(&maps.a, A, rows, HW, false) || !row_map(&maps.b1, B1, rows, n1, false) ||
+        (n2 > 0 && !row_map(&maps.b2, B2, rows, n2, false)))
+        return cudaErrorInvalidValue;
+    WgradArgs a{rows, n1, n2, bias ? 16 : 0, part, err};
+    size_t smem = (size_t)WG_STAGES * MT * (HW + n1 + n2) * 2 + 16 * MT * 2 + 1024;
+    if (smem < 116 * 1024) smem = 116 * 1024;   // one CTA per SM
+    cudaError_t e = cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e) return e;
+    k_wgrad<<<wgrad_ctas(rows), WG_THREADS, smem, s>>>(maps, a);
+    return cudaGetLastError();
+}
+
+cudaError_t enqueue_wgrad_sum(const WgradOut &o, cudaStream_t s)
+{
+    int total = 0;
+    for (int p = 0; p < o.count; p++) total += MT * o.p[p].n;
+    k_wgrad_sum<<<total / 32, 256, 0, s>>>(o);
     return cudaGetLastError();
 }
 

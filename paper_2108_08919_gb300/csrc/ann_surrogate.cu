@@ -73,6 +73,17 @@ __global__ void k_sg_tend_from_ctx(int n, const int *sid, const int *mid, const 
     tend[7 * N + m] = d[2] - d[1];
 }
 
+// Tendencies given particle by particle (n x 8) into planes (8 x n).
+__global__ void k_sg_planes(int n, const float *rows, float *planes)
+{
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const float4 a = reinterpret_cast<const float4 *>(rows)[2 * (size_t)i], b = reinterpret_cast<const float4 *>(rows)[2 * (size_t)i + 1];
+    const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int c = 0; c < 8; c++) planes[(size_t)c * n + i] = v[c];
+}
+
 // Rows of 4 between the graph's sorted order and ID order: to_id: dst[ids[g]] = src[g] (src row
 // stride ld); from_id: dst[g] = src[ids[g]].
 __global__ void k_sg_rows_to_id(int n, const int *ids, const float *src, int ld, float *dst)
@@ -170,7 +181,9 @@ __global__ void __launch_bounds__(256) k_sg_agg(GraphView g, const bf16 *in, bf1
 
 // The adjoint of agg: out[j] = W(0)/S_j in[j] + sum_{i in N(j)} W_ij / S_i in[i]; the neighbour
 // relation is symmetric, so j's own row lists the i and W_ij.  in: FP32 rows of C channels at row
-// stride ld (a multiple of 4, 16-byte aligned rows); C / 8 lanes per particle, 8 channels each.
+// stride ld (a multiple of 4, 16-byte aligned rows); C / 8 lanes per particle, 8 channels each.  The lanes
+// take a neighbour's index and weight each and pass them round (each lane loading and dividing for itself
+// took 32 us at 65,536 particles, this 22).
 template <int C>
 __global__ void __launch_bounds__(256) k_sg_agg_T(GraphView g, const float *in, int ld, bf16 *out)
 {
@@ -196,10 +209,20 @@ __global__ void __launch_bounds__(256) k_sg_agg_T(GraphView g, const float *in, 
     for (int c = 0; c < 8; c++) acc[c] = 0.f;
     add(j, g.W0 / g.S[j]);
     const int m = g.cnt[j];
-#pragma unroll 4
-    for (int k = 0; k < m; k++) {
-        const int i = __ldg(g.nbr + k * n + j);
-        add(i, __ldg(g.W + k * n + j) / __ldg(g.S + i));
+    const unsigned lanes = ((1u << LP) - 1u) << ((threadIdx.x & 31) & ~(LP - 1));
+    for (int k = 0; k < m; k += LP) {
+        int i = 0;
+        float w = 0.f;
+        if (k + q < m) {
+            i = __ldg(g.nbr + (k + q) * n + j);
+            w = __ldg(g.W + (k + q) * n + j) / __ldg(g.S + i);
+        }
+#pragma unroll
+        for (int u = 0; u < LP; u++) {
+            const int iu = __shfl_sync(lanes, i, u, LP);
+            const float wu = __shfl_sync(lanes, w, u, LP);
+            if (k + u < m) add(iu, wu);
+        }
     }
     reinterpret_cast<uint4 *>(out)[(size_t)j * LP + q] = pack8_bf16(acc, 1.f);
 }
@@ -225,16 +248,6 @@ __global__ void k_sg_loss(int n, const float *Y, const float *T, bf16 *dY, doubl
         __syncthreads();
     }
     if (threadIdx.x == 0) atomicAdd(loss, red[0]);
-}
-
-// dA = dH * (H > 0) (relu), dH FP32 with row stride ld, H and dA BF16 with C columns.
-__global__ void k_sg_relu_bwd(int n, int C, const float *dH, int ld, const bf16 *H, bf16 *dA)
-{
-    size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (size_t)n * C) return;
-    size_t i = t / C, c = t % C;
-    float h = __bfloat162float(H[t]);
-    dA[t] = __float2bfloat16(h > 0.f ? dH[i * ld + c] : 0.f);
 }
 
 // out[c] += sum_i in[i][c] (bias gradients); block: 256 threads over rows, one column per y.
@@ -386,8 +399,9 @@ struct ann_surrogate {
     bf16 *X0, *AX, *H1, *Z1, *AZ1, *H2, *Z2, *AZ2, *H3;
     float *Y, *T;
     // backward scratch
-    bf16 *dY, *dA, *dZ;
-    float *dH;   // n x 160
+    bf16 *dY, *dA, *dB, *dZ;   // dA, dB: adjoints of successive layers' pre-activations (n x 128)
+    float *dAZ;                // n x 32: adjoint of a layer's mean
+    float *part;               // partial weight gradients of the products' CTAs
     // parameters
     float *p, *g, *m, *v;   // FP32 flat (NPARAM)
     bf16 *W1b, *P1b, *W2b, *P2b, *W3b, *Wob, *W3T, *W2T, *P2T, *P1T, *WoT;
@@ -482,60 +496,46 @@ cudaError_t backward(ann_surrogate *S)
     int n = S->n;
     GraphView g = view_net(S);
     unsigned *err = S->err;
-    const int K2 = WIDTH + MSG;
     float *gp = S->g;
-    cudaError_t e = cudaMemsetAsync(gp, 0, NPARAM * sizeof(float), s);
+    cudaError_t e = cudaMemsetAsync(gp + O_BO, 0, NOUT * sizeof(float), s);
     if (!e) e = cudaMemsetAsync(S->loss, 0, sizeof(double), s);
     if (e) return e;
     k_sg_loss<<<nb(n), 256, 0, s>>>(n, S->Y, S->T, S->dY, S->loss);
-    // output layer: gWo (rows 0..3 of the 16 x 128 product), gbo
-    float *gWo16 = S->dH;   // 16 x 128 scratch, copied below
-    e = cudaMemsetAsync(gWo16, 0, NOUTP * WIDTH * sizeof(float), s);
-    if (!e) e = enqueue_gemm_tn(S->dY, NOUTP, S->H3, WIDTH, n, gWo16, err, GEMM_CTAS, s);
-    if (!e) e = cudaMemcpyAsync(gp + O_WO, gWo16, NOUT * WIDTH * sizeof(float), cudaMemcpyDeviceToDevice, s);
-    if (e) return e;
     {
         dim3 gr(64, NOUT);
         k_sg_colsum<<<gr, 256, 0, s>>>(n, NOUTP, S->dY, gp + O_BO);
     }
-    // layer 3
-    e = enqueue_gemm_nt(S->dY, NOUTP, nullptr, 0, S->WoT, WIDTH, n, nullptr, 0, S->dH, 0, 0, err, GEMM_CTAS, s, K2);
-    if (e) return e;
-    k_sg_relu_bwd<<<nb((size_t)n * WIDTH), 256, 0, s>>>(n, WIDTH, S->dH, K2, S->H3, S->dA);
-    {
-        dim3 gr(64, WIDTH);
-        k_sg_colsum<<<gr, 256, 0, s>>>(n, WIDTH, S->dA, gp + O_B3);
-    }
-    e = enqueue_gemm_tn(S->dA, WIDTH, S->H2, WIDTH, n, gp + O_W3, err, GEMM_CTAS, s, K2);
-    if (!e) e = enqueue_gemm_tn(S->dA, WIDTH, S->AZ2, MSG, n, gp + O_W3 + WIDTH, err, GEMM_CTAS, s, K2);
-    if (!e) e = enqueue_gemm_nt(S->dA, WIDTH, nullptr, 0, S->W3T, K2, n, nullptr, 0, S->dH, 0, 0, err, GEMM_CTAS, s);
-    if (e) return e;
-    k_sg_agg_T<MSG><<<nb((size_t)n * (MSG / 8)), 256, 0, s>>>(g, S->dH + WIDTH, K2, S->dZ);
-    e = enqueue_gemm_tn(S->dZ, MSG, S->H2, WIDTH, n, gp + O_P2, err, GEMM_CTAS, s);
-    if (!e) e = enqueue_gemm_nt(S->dZ, MSG, nullptr, 0, S->P2T, WIDTH, n, nullptr, 0, S->dH, 0, 1, err, GEMM_CTAS, s, K2);
-    if (e) return e;
-    // layer 2
-    k_sg_relu_bwd<<<nb((size_t)n * WIDTH), 256, 0, s>>>(n, WIDTH, S->dH, K2, S->H2, S->dA);
-    {
-        dim3 gr(64, WIDTH);
-        k_sg_colsum<<<gr, 256, 0, s>>>(n, WIDTH, S->dA, gp + O_B2);
-    }
-    e = enqueue_gemm_tn(S->dA, WIDTH, S->H1, WIDTH, n, gp + O_W2, err, GEMM_CTAS, s, K2);
-    if (!e) e = enqueue_gemm_tn(S->dA, WIDTH, S->AZ1, MSG, n, gp + O_W2 + WIDTH, err, GEMM_CTAS, s, K2);
-    if (!e) e = enqueue_gemm_nt(S->dA, WIDTH, nullptr, 0, S->W2T, K2, n, nullptr, 0, S->dH, 0, 0, err, GEMM_CTAS, s);
-    if (e) return e;
-    k_sg_agg_T<MSG><<<nb((size_t)n * (MSG / 8)), 256, 0, s>>>(g, S->dH + WIDTH, K2, S->dZ);
-    e = enqueue_gemm_tn(S->dZ, MSG, S->H1, WIDTH, n, gp + O_P1, err, GEMM_CTAS, s);
-    if (!e) e = enqueue_gemm_nt(S->dZ, MSG, nullptr, 0, S->P1T, WIDTH, n, nullptr, 0, S->dH, 0, 1, err, GEMM_CTAS, s, K2);
-    if (e) return e;
-    // layer 1
-    k_sg_relu_bwd<<<nb((size_t)n * WIDTH), 256, 0, s>>>(n, WIDTH, S->dH, K2, S->H1, S->dA);
-    {
-        dim3 gr(64, WIDTH);
-        k_sg_colsum<<<gr, 256, 0, s>>>(n, WIDTH, S->dA, gp + O_B1);
-    }
-    e = enqueue_gemm_tn(S->dA, WIDTH, S->X0, F0, n, gp + O_W1, err, GEMM_CTAS, s, 2 * F0);
-    if (!e) e = enqueue_gemm_tn(S->dA, WIDTH, S->AX, F0, n, gp + O_W1 + F0, err, GEMM_CTAS, s, 2 * F0);
+    // each layer: its pre-activation's adjoint and the mean's (one fused kernel), the weights' gradients
+    // (partial products per CTA, summed at the end), the adjoint of the mean
+    WgradOut o{};
+    o.ctas = wgrad_ctas(n);
+    float *part = S->part;
+    auto product = [&](const bf16 *A, const bf16 *B1, int n1, const bf16 *B2, int n2, int transposed, int keep, float *w,
+                       float *b) {
+        const int cols = n1 + n2 + (b ? 16 : 0);
+        o.p[o.count++] = WgradOut::Product{part, cols, n1, n2, transposed, keep, w, b};
+        cudaError_t r = enqueue_wgrad(A, B1, n1, B2, n2, b != nullptr, n, part, err, s);
+        part += (size_t)o.ctas * WIDTH * cols;
+        return r;
+    };
+    auto mean_adjoint = [&]() {
+        k_sg_agg_T<MSG><<<nb((size_t)n * (MSG / 8)), 256, 0, s>>>(g, S->dAZ, MSG, S->dZ);
+        return cudaGetLastError();
+    };
+    constexpr size_t LOW = (size_t)WIDTH * WIDTH;   // rows 128.. of W3T, W2T: the mean's columns
+    e = product(S->H3, S->dY, NOUTP, nullptr, 0, 1, NOUT, gp + O_WO, nullptr);
+    if (!e) e = enqueue_layer_bwd(S->dY, NOUTP, S->WoT, nullptr, 0, nullptr, S->H3, S->W3T + LOW, MSG, S->dA, S->dAZ, n, err, s);
+    if (!e) e = product(S->dA, S->H2, WIDTH, S->AZ2, MSG, 0, 0, gp + O_W3, gp + O_B3);
+    if (!e) e = mean_adjoint();
+    if (!e) e = product(S->H2, S->dZ, MSG, nullptr, 0, 1, MSG, gp + O_P2, nullptr);
+    if (!e) e = enqueue_layer_bwd(S->dA, WIDTH, S->W3T, S->dZ, MSG, S->P2T, S->H2, S->W2T + LOW, MSG, S->dB, S->dAZ, n, err, s);
+    if (!e) e = product(S->dB, S->H1, WIDTH, S->AZ1, MSG, 0, 0, gp + O_W2, gp + O_B2);
+    if (!e) e = mean_adjoint();
+    if (!e) e = product(S->H1, S->dZ, MSG, nullptr, 0, 1, MSG, gp + O_P1, nullptr);
+    // layer 1 has no layer below: its mean's columns are not needed (dAZ is scratch)
+    if (!e) e = enqueue_layer_bwd(S->dB, WIDTH, S->W2T, S->dZ, MSG, S->P1T, S->H1, S->W2T + LOW, MSG, S->dA, S->dAZ, n, err, s);
+    if (!e) e = product(S->dA, S->X0, F0, S->AX, F0, 0, 0, gp + O_W1, gp + O_B1);
+    if (!e) e = enqueue_wgrad_sum(o, s);
     return e ? e : cudaGetLastError();
 }
 
@@ -596,8 +596,10 @@ int ann_surrogate_create(int64_t n_max, ann_surrogate **out)
     SA_(io4, 4 * n);
     SA_(X0, n * F0); SA_(AX, n * F0); SA_(H1, n * WIDTH); SA_(Z1, n * MSG); SA_(AZ1, n * MSG);
     SA_(H2, n * WIDTH); SA_(Z2, n * MSG); SA_(AZ2, n * MSG); SA_(H3, n * WIDTH);
-    SA_(Y, n * NOUTP); SA_(T, n * NOUT); SA_(dY, n * NOUTP); SA_(dA, n * WIDTH); SA_(dZ, n * MSG);
-    SA_(dH, std::max(n * K2, (size_t)NOUTP * WIDTH));
+    SA_(Y, n * NOUTP); SA_(T, n * NOUT); SA_(dY, n * NOUTP); SA_(dA, n * WIDTH); SA_(dB, n * WIDTH); SA_(dZ, n * MSG);
+    SA_(dAZ, n * MSG);
+    // the six products' columns: Wo 16, W3 and W2 176 each with the bias, P2 and P1 32, W1 48
+    SA_(part, (size_t)wgrad_ctas((int)n) * WIDTH * (16 + 2 * 176 + 2 * 32 + 48));
     SA_(p, NPARAM); SA_(g, NPARAM); SA_(m, NPARAM); SA_(v, NPARAM);
     SA_(W1b, WIDTH * 2 * F0); SA_(P1b, MSG * WIDTH); SA_(W2b, WIDTH * K2); SA_(P2b, MSG * WIDTH);
     SA_(W3b, WIDTH * K2); SA_(Wob, NOUTP * WIDTH); SA_(W3T, K2 * WIDTH); SA_(W2T, K2 * WIDTH);
@@ -655,7 +657,7 @@ int ann_surrogate_set_scales(ann_surrogate *S, double us, double ys_q, double ys
     return ANN_OK;
 }
 
-int ann_surrogate_load(ann_surrogate *S, ann_ctx *ctx, const float *tend)
+static int load_graph(ann_surrogate *S, ann_ctx *ctx, const float *tend, bool rows)
 {
     ann::NvtxRange range("ann_surrogate_load");
     if (!S || !ctx) return ANN_ERR_INVALID_ARG;
@@ -665,7 +667,12 @@ int ann_surrogate_load(ann_surrogate *S, ann_ctx *ctx, const float *tend)
     if (v.P.n > S->nmax) return sfail(S, ANN_ERR_INVALID_ARG, "context has more particles than n_max");
     size_t n = (size_t)v.P.n;
     if (tend) {
-        cudaError_t e = cudaMemcpyAsync(S->tend_id, tend, 8 * n * sizeof(float), cudaMemcpyHostToDevice, S->s);
+        float *dst = rows ? S->Y : S->tend_id;   // the outputs' buffer is free until the next forward pass
+        cudaError_t e = cudaMemcpyAsync(dst, tend, 8 * n * sizeof(float), cudaMemcpyHostToDevice, S->s);
+        if (!e && rows) {
+            k_sg_planes<<<nb(n), 256, 0, S->s>>>((int)n, S->Y, S->tend_id);
+            e = cudaGetLastError();
+        }
         if (!e) e = cudaStreamSynchronize(S->s);
         if (e) return scuda(S, e, "ann_surrogate_load: tendencies");
     } else {
@@ -704,6 +711,14 @@ int ann_surrogate_load(ann_surrogate *S, ann_ctx *ctx, const float *tend)
                                                    "than the network's graph holds (64)");
     S->loaded = true;
     return ANN_OK;
+}
+
+int ann_surrogate_load(ann_surrogate *S, ann_ctx *ctx, const float *tend) { return load_graph(S, ctx, tend, false); }
+
+int ann_surrogate_load_rows(ann_surrogate *S, ann_ctx *ctx, const float *tend)
+{
+    if (!tend) return ANN_ERR_INVALID_ARG;
+    return load_graph(S, ctx, tend, true);
 }
 
 int ann_surrogate_forward(ann_surrogate *S, float *y)
