@@ -36,6 +36,30 @@ __device__ __forceinline__ bool in_box(double x, long long bitsL)
     return bx >= 0 && bx < bitsL;
 }
 
+// Conversions between FP32 and FP64 in integer arithmetic, bit for bit those of the hardware's
+// instructions.  A conversion runs on the FP64 pipe, at 1/64 of the FP32 rate, and a kernel that walks
+// the particles once is bound by that pipe: the predictor spent 8 of its 14 FP64 operations a particle
+// on conversions (k_predict at 1024^2 particles: 38 us with the instructions, 31 so; k_keys 31 and 21).  Zeros and normal values are done here; FP32 subnormals, overflow, infinity and NaN, which need
+// more than shifts, go to the instruction.
+__device__ __forceinline__ double widen(float f)
+{
+    const uint32_t u = __float_as_uint(f);
+    if (((u & 0x7f800000u) - 0x00800000u) < 0x7f000000u)
+        return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+    return (u << 1) == 0u ? __hiloint2double((int)u, 0) : (double)f;
+}
+
+__device__ __forceinline__ float narrow(double d)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(d);
+    const unsigned long long a = (unsigned long long)__double_as_longlong(d) & 0x7fffffffffffffffull;
+    // 2^-126 <= |d| < 2^127: drop 29 bits of the fraction, to nearest, ties to even, and re-bias
+    if (((hi & 0x7ff00000u) - 0x38100000u) < 0x0fd00000u)
+        return __uint_as_float((hi & 0x80000000u) |
+                               ((uint32_t)((a + 0x0fffffffull + ((a >> 29) & 1ull)) >> 29) - 0xc0000000u));
+    return a == 0ull ? __uint_as_float(hi) : (float)d;
+}
+
 // Two-lane FP32 arithmetic (one instruction issues both lanes, each lane rounded as the scalar
 // operation).  The pair passes are issue-bound, and their x/y arithmetic pairs up naturally.
 __device__ __forceinline__ float2 f2(float x, float y) { return make_float2(x, y); }

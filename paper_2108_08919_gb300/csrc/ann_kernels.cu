@@ -202,8 +202,8 @@ __device__ __forceinline__ const T &slot_at(const T *base, int o)
 // exact in both precisions; lo = o - hi, exact in FP64, then rounded to FP32.
 __device__ __forceinline__ float2 split_offset(double o, const DevParams &P)
 {
-    float hi = rintf((float)o * P.iqf) * P.qf;
-    return make_float2(hi, (float)(o - (double)hi));
+    float hi = rintf(narrow(o) * P.iqf) * P.qf;
+    return make_float2(hi, narrow(o - widen(hi)));
 }
 
 __global__ void __launch_bounds__(256, 8) k_predict(DevParams P, Bufs b)
@@ -220,8 +220,8 @@ __global__ void __launch_bounds__(256, 8) k_predict(DevParams P, Bufs b)
         float ux = in.ux[i] + P.half_dt * in.ax[i];
         float uy = in.uy[i] + P.half_dt * in.ay[i];
         // FP64 work is kept to what the positions need: GB300 issues FP64 at 1/64 of FP32.
-        double x = in.x[i] + (double)(P.half_dt * ux);
-        double y = in.y[i] + (double)(P.half_dt * uy);
+        double x = in.x[i] + widen(P.half_dt * ux);
+        double y = in.y[i] + widen(P.half_dt * uy);
         if (!(in_box(x, P.bitsL) && in_box(y, P.bitsL))) {   // rare: crossed a face, or not finite
             int kx = wrap_count(x, P.L), ky = wrap_count(y, P.L);
             x = x + 0.0;
@@ -1222,8 +1222,8 @@ __global__ void BOUNDS_D k_pass_d(DevParams P, Bufs b)
             apy = sc_ * sdy;
         }
         float stepx = P.half_dt * unx + apx, stepy = P.half_dt * uny + apy;
-        double xn = mxi + (double)stepx;
-        double yn = myi + (double)stepy;
+        double xn = mxi + widen(stepx);
+        double yn = myi + widen(stepy);
         if (!(in_box(xn, P.bitsL) && in_box(yn, P.bitsL))) {   // rare: re-insert (Eq. 30)
             int kx = wrap_count(xn, P.L), ky = wrap_count(yn, P.L);
             xn = xn + 0.0;

