@@ -181,6 +181,15 @@ int lanes_for(int tiles)
     return lanes;
 }
 
+// Threads per block of the pair passes.  A cell is at least 3h (1 + skin) wide, 3.98 spacings at h = 1.3 dx,
+// so that a tile holds 250 to 260 particles: with 256 threads about half of the tiles go round their
+// particles twice, the second time for a handful.  Where all tiles run at once (4 to 5 blocks an SM) the
+// slowest tile is the pass: one round of 288 threads, at 4 blocks an SM instead of 5, took (us a step)
+// 104 -> 89 at 441 tiles (333^2, conservative), 71 -> 67 at 256 (256^2), 142 -> 139 at 1,024, 189 -> 184
+// at 1,444; with 4,225 (1024^2) the waves hide the second round, and the fifth block is worth more:
+// 447 -> 456, and 6,129 -> 6,290 at 4096^2.  320 threads: 90 at 441 tiles, 465 at 4,225.
+int threads_for(int tiles) { return tiles <= 1520 ? PT_FEW : PT; }   // ten tiles an SM
+
 DevParams make_dev(const ann_params &p)
 {
     DevParams d{};
@@ -189,6 +198,7 @@ DevParams make_dev(const ann_params &p)
     d.ncell = d.nc * d.nc;
     d.tiles = (d.nc + TILE - 1) / TILE;
     d.lanes = lanes_for(d.tiles * d.tiles);
+    d.threads = threads_for(d.tiles * d.tiles);
     d.apd = p.apd;
     d.conservative = p.momentum_mode == ANN_MOMENTUM_CONSERVATIVE;
     d.qnew = p.q_new_in_momentum;

@@ -30,6 +30,7 @@ constexpr int MAXN = 128;             // neighbours per particle (ANN_MAX_NEIGHB
 constexpr int MAXN2H = 64;            // neighbours closer than 2h kept in the surrogate's graph
 constexpr int MAXC = 64;              // particles per cell (ANN_MAX_PER_CELL)
 constexpr int PT = 256;               // threads per pair-pass block
+constexpr int PT_FEW = 288;           // the same in a box of few tiles (threads_for)
 constexpr int NKERNELS = 10;
 // Candidate ("Verlet") lists hold every pair within 3h (1 + SKIN) at the last re-sort; they stay
 // valid until some particle has moved SKIN/2 * 3h.  Cells are at least 3h (1 + SKIN) wide.
@@ -51,6 +52,7 @@ enum : uint32_t {
 struct DevParams {
     int n, nc, ncell, tiles;
     int lanes;             // lanes per particle of passes A to D (1, 2, 4 or 8), by the tile count
+    int threads;           // threads per block of the pair passes (PT or PT_FEW), by the tile count
     int apd, conservative, qnew, record, elastic;
     double L, cell, inv_cell, R2, dt_d, half_dt_d;
     double q;              // power-of-two grid of the "hi" coordinate part: cell / q in [2^12, 2^13)

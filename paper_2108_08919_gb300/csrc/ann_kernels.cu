@@ -475,10 +475,10 @@ __device__ __forceinline__ bool in_support(float r2, const DevParams &P, const B
 constexpr uint32_t SLOT_OFF_MASK = (HCAP - 1) << 4;
 static_assert(((HCAP - 1) << 4) <= 0xffff, "slot offsets must fit 16 bits");
 
-constexpr int SMEM_A = HCAP * (16 + 4 + 1) + MAXV * PT * 2;
+constexpr int smem_a(int T) { return HCAP * (16 + 4 + 1) + MAXV * T * 2; }
 
-template <bool FROM_REF>
-__global__ void __launch_bounds__(PT) k_pass_a_resort(DevParams P, Bufs b)
+template <bool FROM_REF, int T>
+__global__ void __launch_bounds__(T) k_pass_a_resort(DevParams P, Bufs b)
 {
     if (!FROM_REF && !resorting(b)) return;
     __shared__ TileShared ts;
@@ -487,10 +487,10 @@ __global__ void __launch_bounds__(PT) k_pass_a_resort(DevParams P, Bufs b)
     const float2 *phi = reinterpret_cast<const float2 *>(dsm);   // hi parts: phi[2 j] = pos[j].xy
     int *sg = reinterpret_cast<int *>(pos + HCAP);
     uint16_t *lst = reinterpret_cast<uint16_t *>(sg + HCAP);
-    unsigned char *shc = reinterpret_cast<unsigned char *>(lst + MAXV * PT);
-    Tile T;
-    if (!tile_begin(P, b, ts, T)) return;
-    for (int t = threadIdx.x; t < T.H; t += PT) {
+    unsigned char *shc = reinterpret_cast<unsigned char *>(lst + MAXV * T);
+    Tile tile;
+    if (!tile_begin(P, b, ts, tile)) return;
+    for (int t = threadIdx.x; t < tile.H; t += T) {
         const SlotInfo s = slot_info<FROM_REF>(P, b, ts, t);
         pos[t] = s.e;
         sg[t] = s.g;
@@ -498,8 +498,8 @@ __global__ void __launch_bounds__(PT) k_pass_a_resort(DevParams P, Bufs b)
     }
     __syncthreads();
     if (!FROM_REF && first_thread()) atomicAdd(b.resorts, 1u);
-    uint16_t *my = lst + threadIdx.x;   // this thread's list column, stride PT
-    for (int q = threadIdx.x; q < T.Ni; q += PT) {
+    uint16_t *my = lst + threadIdx.x;   // this thread's list column, stride T
+    for (int q = threadIdx.x; q < tile.Ni; q += T) {
         int si = inner_slot(ts, q);
         const int h = shc[si];
         float4 pi = pos[si];
@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(PT) k_pass_a_resort(DevParams P, Bufs b)
                 float2 pj = phi[2 * j];
                 float dx = pi.x - pj.x, dy = pi.y - pj.y;
                 bool in = (dx * dx + dy * dy < P.R2c) & (j != si);
-                my[min(cnt, MAXV - 1) * PT] = (uint16_t)j;
+                my[min(cnt, MAXV - 1) * T] = (uint16_t)j;
                 cnt += in;
             }
         }
@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(PT) k_pass_a_resort(DevParams P, Bufs b)
         float sw = P.W0;
         int cv = 0, nn = 0, nlow = 0;
         for (int k = 0; k < cnt; k++) {
-            int j = my[k * PT];   // slot (the coarse scan stores slots)
+            int j = my[k * T];   // slot (the coarse scan stores slots)
             float2 d = pair_d(pi, pos[j]);
             float r2 = len2(d);
             bool cand = r2 < P.R2v;
@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(PT) k_pass_a_resort(DevParams P, Bufs b)
                 nn += in;
             }
             // byte offset of the slot; bit 0 (free: offsets are multiples of 16) carries the support bit
-            my[cv * PT] = (uint16_t)((j << 4) | (int)in);
+            my[cv * T] = (uint16_t)((j << 4) | (int)in);
             nlow += cand & (j < si);
             cv += cand;
         }
@@ -542,7 +542,7 @@ __global__ void __launch_bounds__(PT) k_pass_a_resort(DevParams P, Bufs b)
         // si and wraps around.  The threads of a warp hold consecutive slots, so at each step of
         // their walks they load mostly distinct, consecutive slots, which spreads the staged loads
         // of the pair passes over the shared-memory banks (ascending order: ~2x the bank conflicts).
-        auto at = [&](int k) { return (uint32_t)my[(k + nlow < cv ? k + nlow : k + nlow - cv) * PT]; };
+        auto at = [&](int k) { return (uint32_t)my[(k + nlow < cv ? k + nlow : k + nlow - cv) * T]; };
         uint2 *out = b.vnbr + gi;
         for (int k = 0; k < cv; k += 4) {
             uint32_t s0 = at(k);
@@ -597,27 +597,13 @@ __global__ void __launch_bounds__(PT) k_pass_a_resort(DevParams P, Bufs b)
 #ifndef ANN_PF_D
 #define ANN_PF_D 1
 #endif
-#define ANN_BOUNDS(minb) __launch_bounds__(PT, (minb) > 0 ? (minb) : 1)
-#if ANN_MINB_A > 0
-#define BOUNDS_A ANN_BOUNDS(LP > 1 ? ANN_MINB_L : ANN_MINB_A)
-#else
-#define BOUNDS_A __launch_bounds__(PT)
-#endif
-#if ANN_MINB_B > 0
-#define BOUNDS_B ANN_BOUNDS(LP > 1 ? ANN_MINB_L : ANN_MINB_B)
-#else
-#define BOUNDS_B __launch_bounds__(PT)
-#endif
-#if ANN_MINB_C > 0
-#define BOUNDS_C ANN_BOUNDS(LP > 1 ? ANN_MINB_L : ANN_MINB_C)
-#else
-#define BOUNDS_C __launch_bounds__(PT)
-#endif
-#if ANN_MINB_D > 0
-#define BOUNDS_D ANN_BOUNDS(LP > 1 ? ANN_MINB_L : ANN_MINB_D)
-#else
-#define BOUNDS_D __launch_bounds__(PT)
-#endif
+// T threads (PT, or PT_FEW where the tiles are few: see threads_for), with fewer blocks of the wider kind
+#define ANN_BOUNDS(minb) \
+    __launch_bounds__(T, T > PT ? ANN_MINB_L : (minb) > 0 ? (minb) : 1)
+#define BOUNDS_A ANN_BOUNDS(ANN_MINB_A)
+#define BOUNDS_B ANN_BOUNDS(ANN_MINB_B)
+#define BOUNDS_C ANN_BOUNDS(ANN_MINB_C)
+#define BOUNDS_D ANN_BOUNDS(ANN_MINB_D)
 
 // Visit the candidates of particle gi (c of them, four per 64-bit list word) in order, keeping the
 // next PF words in flight while the current ones are processed: fn(byte offset of the slot,
@@ -687,11 +673,11 @@ __device__ __forceinline__ void for_each_candidate(const DevParams &P, const Buf
 // Lanes per particle (P.lanes: 1, 2, 4 or 8, the template argument LP of the passes).  A box of few
 // tiles leaves the GPU idle with one block per tile and one thread per particle: 64^2 has 16 tiles for
 // 152 SMs, and a thread's walk of 46 candidates is most of a pass.  There LP blocks share a tile (each
-// stages the whole halo and takes PT / LP of its particles) and LP lanes a particle's candidate words.
-template <int LP>
+// stages the whole halo and takes its share of the particles, T / LP at a time) and LP lanes a particle's candidate words.
+template <int LP, int T>
 __device__ __forceinline__ int first_particle()
 {
-    return (int)((blockIdx.x % LP) * PT + threadIdx.x) / LP;
+    return (int)((blockIdx.x % LP) * T + threadIdx.x) / LP;
 }
 
 // The lanes' sums; every lane of the particle gets the total (a no-op for one lane).
@@ -735,7 +721,7 @@ __device__ __forceinline__ bool writes()
 
 constexpr int SMEM_AF = HCAP * (16 + 4);
 
-template <int LP>
+template <int LP, int T>
 __global__ void BOUNDS_A k_pass_a_filter(DevParams P, Bufs b)
 {
     if (resorting(b)) return;
@@ -743,15 +729,15 @@ __global__ void BOUNDS_A k_pass_a_filter(DevParams P, Bufs b)
     extern __shared__ __align__(16) unsigned char dsm[];
     float4 *pos = reinterpret_cast<float4 *>(dsm);
     int *sg = reinterpret_cast<int *>(pos + HCAP);
-    Tile T;
-    if (!tile_begin<LP>(P, b, ts, T)) return;
-    for (int t = threadIdx.x; t < T.H; t += PT) {
+    Tile tile;
+    if (!tile_begin<LP>(P, b, ts, tile)) return;
+    for (int t = threadIdx.x; t < tile.H; t += T) {
         SlotInfo s = slot_info(P, b, ts, t);
         pos[t] = s.e;
         sg[t] = s.g;
     }
     __syncthreads();
-    for (int q = first_particle<LP>(); q < T.Ni; q += PT) {
+    for (int q = first_particle<LP, T>(); q < tile.Ni; q += T) {
         int si = inner_slot(ts, q);
         int gi = sg[si];
         float4 pi = pos[si];
@@ -824,7 +810,7 @@ __global__ void BOUNDS_A k_pass_a_filter(DevParams P, Bufs b)
 
 constexpr int SMEM_B = HCAP * (16 + 16 + 4 + 4);
 
-template <bool QOLD, int LP>
+template <bool QOLD, int LP, int T>
 __global__ void BOUNDS_B k_pass_b(DevParams P, Bufs b)
 {
     __shared__ TileShared ts;
@@ -833,10 +819,10 @@ __global__ void BOUNDS_B k_pass_b(DevParams P, Bufs b)
     float4 *sb = sp + HCAP;                           // (ux, uy, q11, q12): two-lane pairs in place
     float *sv = reinterpret_cast<float *>(sb + HCAP); // V
     int *sg = reinterpret_cast<int *>(sv + HCAP);
-    Tile T;
-    if (!tile_begin<LP>(P, b, ts, T)) return;
+    Tile tile;
+    if (!tile_begin<LP>(P, b, ts, tile)) return;
     if (first_thread()) *b.rebuild = 0u;   // both pass A kernels have run
-    for (int t = threadIdx.x; t < T.H; t += PT) {
+    for (int t = threadIdx.x; t < tile.H; t += T) {
         SlotInfo s = slot_info(P, b, ts, t);
         sp[t] = s.e;
         sb[t] = b.mu4[s.g];
@@ -844,7 +830,7 @@ __global__ void BOUNDS_B k_pass_b(DevParams P, Bufs b)
         sg[t] = s.g;
     }
     __syncthreads();
-    for (int q = first_particle<LP>(); q < T.Ni; q += PT) {
+    for (int q = first_particle<LP, T>(); q < tile.Ni; q += T) {
         int si = inner_slot(ts, q);
         int gi = sg[si];
         float4 pi = sp[si], bi = sb[si];
@@ -968,7 +954,7 @@ __global__ void BOUNDS_B k_pass_b(DevParams P, Bufs b)
 // the elastic stress tile exists only in the instantiations that read it
 constexpr int smem_c(bool el) { return HCAP * (16 + 16 + (el ? 16 : 0) + 4); }
 
-template <bool QNEW, bool EL, int LP>
+template <bool QNEW, bool EL, int LP, int T>
 __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
 {
     __shared__ TileShared ts;
@@ -977,10 +963,10 @@ __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
     float4 *sb = sp + HCAP;                            // (V, drho_half, q11^{n+1}, q12^{n+1})
     float4 *se = sb + HCAP;                            // elastic stress (11, 12, 22, -)
     int *sg = reinterpret_cast<int *>(se + (EL ? HCAP : 0));
-    Tile T;
-    if (!tile_begin<LP>(P, b, ts, T)) return;
+    Tile tile;
+    if (!tile_begin<LP>(P, b, ts, tile)) return;
     const StateSet out = state_out(b);   // Q^{n+1} (pass B)
-    for (int t = threadIdx.x; t < T.H; t += PT) {
+    for (int t = threadIdx.x; t < tile.H; t += T) {
         SlotInfo s = slot_info(P, b, ts, t);
         sp[t] = s.e;
         sb[t] = b.cr[s.g];   // (V, delta_half, Q^{n+1}); pass C reads Q^{n+1} only with QNEW
@@ -995,7 +981,7 @@ __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
     if (P.dt_check && first_thread() &&
         (P.dt > P.dt_static || P.dt * (c0 + umax) * P.inv_h > 0.25f))
         atomicOr(b.err, EB_CFL);
-    for (int q = first_particle<LP>(); q < T.Ni; q += PT) {
+    for (int q = first_particle<LP, T>(); q < tile.Ni; q += T) {
         int si = inner_slot(ts, q);
         int gi = sg[si];
         float4 pi = sp[si], bi = sb[si];
@@ -1083,7 +1069,7 @@ __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
 // (the (q11, q12)/rho^2 tile exists in the conservative mode only, Pi/rho^2 with the elastic stress)
 constexpr int smem_d(bool cons, bool el) { return HCAP * (16 + 16 + (cons ? 8 : 0) + (cons && el ? 16 : 0) + 4); }
 
-template <bool CONS, bool EL, int LP>
+template <bool CONS, bool EL, int LP, int T>
 __global__ void BOUNDS_D k_pass_d(DevParams P, Bufs b)
 {
     __shared__ TileShared ts;
@@ -1095,11 +1081,11 @@ __global__ void BOUNDS_D k_pass_d(DevParams P, Bufs b)
     int *sg = reinterpret_cast<int *>(se + ((CONS && EL) ? HCAP : 0));
     // the step's output set: Q^{n+1} (pass B) in, the new state out; k_commit of the next step (or
     // the host) commits it if no error has been raised by then
-    Tile T;
-    if (!tile_begin<LP>(P, b, ts, T)) return;
+    Tile tile;
+    if (!tile_begin<LP>(P, b, ts, tile)) return;
     if (first_thread()) b.ctl[CTL_PENDING] = 1u;
     const StateSet out = state_out(b);
-    for (int t = threadIdx.x; t < T.H; t += PT) {
+    for (int t = threadIdx.x; t < tile.H; t += T) {
         SlotInfo s = slot_info(P, b, ts, t);
         sp[t] = s.e;
         if (CONS) {
@@ -1123,7 +1109,7 @@ __global__ void BOUNDS_D k_pass_d(DevParams P, Bufs b)
     }
     __syncthreads();
     if (first_thread()) *b.maxu = 0u;   // pass C has consumed it
-    for (int q = first_particle<LP>(); q < T.Ni; q += PT) {
+    for (int q = first_particle<LP, T>(); q < tile.Ni; q += T) {
         int si = inner_slot(ts, q);
         int gi = sg[si];
         float4 pi = sp[si], bi = sb[si];
@@ -1575,46 +1561,46 @@ cudaError_t allow_smem(F *f, int bytes)
     return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
-template <int LP>
+template <int LP, int T>
 cudaError_t prepare_passes()
 {
     cudaError_t e;
-    if ((e = allow_smem(k_pass_a_filter<LP>, SMEM_AF))) return e;
-    if ((e = allow_smem(k_pass_b<false, LP>, SMEM_B))) return e;
-    if ((e = allow_smem(k_pass_b<true, LP>, SMEM_B))) return e;
-    if ((e = allow_smem(k_pass_c<false, false, LP>, smem_c(false)))) return e;
-    if ((e = allow_smem(k_pass_c<true, false, LP>, smem_c(false)))) return e;
-    if ((e = allow_smem(k_pass_c<false, true, LP>, smem_c(true)))) return e;
-    if ((e = allow_smem(k_pass_c<true, true, LP>, smem_c(true)))) return e;
-    if ((e = allow_smem(k_pass_d<false, false, LP>, smem_d(false, false)))) return e;
-    if ((e = allow_smem(k_pass_d<true, false, LP>, smem_d(true, false)))) return e;
-    if ((e = allow_smem(k_pass_d<false, true, LP>, smem_d(false, true)))) return e;
-    return allow_smem(k_pass_d<true, true, LP>, smem_d(true, true));
+    if ((e = allow_smem(k_pass_a_filter<LP, T>, SMEM_AF))) return e;
+    if ((e = allow_smem(k_pass_b<false, LP, T>, SMEM_B))) return e;
+    if ((e = allow_smem(k_pass_b<true, LP, T>, SMEM_B))) return e;
+    if ((e = allow_smem(k_pass_c<false, false, LP, T>, smem_c(false)))) return e;
+    if ((e = allow_smem(k_pass_c<true, false, LP, T>, smem_c(false)))) return e;
+    if ((e = allow_smem(k_pass_c<false, true, LP, T>, smem_c(true)))) return e;
+    if ((e = allow_smem(k_pass_c<true, true, LP, T>, smem_c(true)))) return e;
+    if ((e = allow_smem(k_pass_d<false, false, LP, T>, smem_d(false, false)))) return e;
+    if ((e = allow_smem(k_pass_d<true, false, LP, T>, smem_d(true, false)))) return e;
+    if ((e = allow_smem(k_pass_d<false, true, LP, T>, smem_d(false, true)))) return e;
+    return allow_smem(k_pass_d<true, true, LP, T>, smem_d(true, true));
 }
 
 // Pass k (6 to 9) with LP lanes per particle.
-template <int LP>
+template <int LP, int T>
 void launch_pass(int k, const DevParams &P, const Bufs &b, cudaStream_t s)
 {
     const dim3 nt(P.tiles * LP, P.tiles);
     const bool el = P.elastic && !P.conservative;   // the paper momentum takes div Pi from pass C
     switch (k) {
-    case 6: k_pass_a_filter<LP><<<nt, PT, SMEM_AF, s>>>(P, b); break;
+    case 6: k_pass_a_filter<LP, T><<<nt, T, SMEM_AF, s>>>(P, b); break;
     case 7:
-        if (P.qnew) k_pass_b<false, LP><<<nt, PT, SMEM_B, s>>>(P, b);
-        else k_pass_b<true, LP><<<nt, PT, SMEM_B, s>>>(P, b);
+        if (P.qnew) k_pass_b<false, LP, T><<<nt, T, SMEM_B, s>>>(P, b);
+        else k_pass_b<true, LP, T><<<nt, T, SMEM_B, s>>>(P, b);
         break;
     case 8:
-        if (P.qnew && el) k_pass_c<true, true, LP><<<nt, PT, smem_c(true), s>>>(P, b);
-        else if (P.qnew) k_pass_c<true, false, LP><<<nt, PT, smem_c(false), s>>>(P, b);
-        else if (el) k_pass_c<false, true, LP><<<nt, PT, smem_c(true), s>>>(P, b);
-        else k_pass_c<false, false, LP><<<nt, PT, smem_c(false), s>>>(P, b);
+        if (P.qnew && el) k_pass_c<true, true, LP, T><<<nt, T, smem_c(true), s>>>(P, b);
+        else if (P.qnew) k_pass_c<true, false, LP, T><<<nt, T, smem_c(false), s>>>(P, b);
+        else if (el) k_pass_c<false, true, LP, T><<<nt, T, smem_c(true), s>>>(P, b);
+        else k_pass_c<false, false, LP, T><<<nt, T, smem_c(false), s>>>(P, b);
         break;
     case 9:
-        if (P.conservative && P.elastic) k_pass_d<true, true, LP><<<nt, PT, smem_d(true, true), s>>>(P, b);
-        else if (P.conservative) k_pass_d<true, false, LP><<<nt, PT, smem_d(true, false), s>>>(P, b);
-        else if (P.elastic) k_pass_d<false, true, LP><<<nt, PT, smem_d(false, true), s>>>(P, b);
-        else k_pass_d<false, false, LP><<<nt, PT, smem_d(false, false), s>>>(P, b);
+        if (P.conservative && P.elastic) k_pass_d<true, true, LP, T><<<nt, T, smem_d(true, true), s>>>(P, b);
+        else if (P.conservative) k_pass_d<true, false, LP, T><<<nt, T, smem_d(true, false), s>>>(P, b);
+        else if (P.elastic) k_pass_d<false, true, LP, T><<<nt, T, smem_d(false, true), s>>>(P, b);
+        else k_pass_d<false, false, LP, T><<<nt, T, smem_d(false, false), s>>>(P, b);
         break;
     }
 }
@@ -1624,12 +1610,14 @@ void launch_pass(int k, const DevParams &P, const Bufs &b, cudaStream_t s)
 cudaError_t prepare_kernels()
 {
     cudaError_t e;
-    if ((e = allow_smem(k_pass_a_resort<false>, SMEM_A))) return e;
-    if ((e = allow_smem(k_pass_a_resort<true>, SMEM_A))) return e;
-    if ((e = prepare_passes<1>())) return e;
-    if ((e = prepare_passes<2>())) return e;
-    if ((e = prepare_passes<4>())) return e;
-    return prepare_passes<8>();
+    if ((e = allow_smem(k_pass_a_resort<false, PT>, smem_a(PT)))) return e;
+    if ((e = allow_smem(k_pass_a_resort<false, PT_FEW>, smem_a(PT_FEW)))) return e;
+    if ((e = allow_smem(k_pass_a_resort<true, PT>, smem_a(PT)))) return e;
+    if ((e = prepare_passes<1, PT>())) return e;
+    if ((e = prepare_passes<1, PT_FEW>())) return e;
+    if ((e = prepare_passes<2, PT_FEW>())) return e;
+    if ((e = prepare_passes<4, PT_FEW>())) return e;
+    return prepare_passes<8, PT_FEW>();
 }
 
 // Kernel k of the step on stream s (see kNames).
@@ -1643,12 +1631,16 @@ cudaError_t launch_kernel(int k, const DevParams &P, const Bufs &b, cudaStream_t
     case 2: k_scan<<<P.nsblk, 1024, 0, s>>>(P, b); break;
     case 3: k_scatter<<<nb, 256, 0, s>>>(P, b); break;
     case 4: k_cell_order<<<blocks_for(P.ncell, 8), 256, 0, s>>>(P, b); break;
-    case 5: k_pass_a_resort<false><<<nt, PT, SMEM_A, s>>>(P, b); break;
+    case 5:
+        if (P.threads == PT_FEW) k_pass_a_resort<false, PT_FEW><<<nt, PT_FEW, smem_a(PT_FEW), s>>>(P, b);
+        else k_pass_a_resort<false, PT><<<nt, PT, smem_a(PT), s>>>(P, b);
+        break;
     case 6: case 7: case 8: case 9:
-        if (P.lanes == 8) launch_pass<8>(k, P, b, s);
-        else if (P.lanes == 4) launch_pass<4>(k, P, b, s);
-        else if (P.lanes == 2) launch_pass<2>(k, P, b, s);
-        else launch_pass<1>(k, P, b, s);
+        if (P.lanes == 8) launch_pass<8, PT_FEW>(k, P, b, s);
+        else if (P.lanes == 4) launch_pass<4, PT_FEW>(k, P, b, s);
+        else if (P.lanes == 2) launch_pass<2, PT_FEW>(k, P, b, s);
+        else if (P.threads == PT_FEW) launch_pass<1, PT_FEW>(k, P, b, s);
+        else launch_pass<1, PT>(k, P, b, s);
         break;
     default: return cudaErrorInvalidValue;
     }
@@ -1684,7 +1676,7 @@ cudaError_t enqueue_search(const DevParams &P, const Bufs &b, cudaStream_t s)
 
 cudaError_t enqueue_candidates_from_ref(const DevParams &P, const Bufs &b, cudaStream_t s)
 {
-    k_pass_a_resort<true><<<dim3(P.tiles, P.tiles), PT, SMEM_A, s>>>(P, b);
+    k_pass_a_resort<true, PT><<<dim3(P.tiles, P.tiles), PT, smem_a(PT), s>>>(P, b);
     return cudaGetLastError();
 }
 
