@@ -2,6 +2,8 @@
 #include "../../include/ann.h"
 #include "ann_device.cuh"
 
+#include <cudaTypedefs.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -698,6 +700,51 @@ __global__ void k_get_state_mapped(Bufs b, int n, const int *inv, double *x, dou
     if (ay) ay[i] = b.say[g];
 }
 
+// The fields of the state in particle order (slot g is particle sid[g]) into the nine arrays of d: the two
+// positions, then the seven FP32 fields (NULL skipped).  One pass for all: a launch per field reads the
+// slots' particles each time (6.5 us a field at 1M particles; all nine here 18).
+struct StateDst {
+    double *x, *y;
+    float *f[7];   // ux, uy, q11, q12, drho, ax, ay
+};
+
+__global__ void __launch_bounds__(256) k_get_state(Bufs b, int n, StateDst d)
+{
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= n) return;
+    const int i = b.sid[g];
+    const float *src[7] = {b.sux, b.suy, b.sq11, b.sq12, b.sdr, b.sax, b.say};
+    if (d.x) d.x[i] = b.sx[g];
+    if (d.y) d.y[i] = b.sy[g];
+#pragma unroll
+    for (int k = 0; k < 7; k++)
+        if (d.f[k]) d.f[k][i] = src[k][g];
+}
+
+// Whether a kernel may write `bytes` at p instead of a copy: device memory of the current device that one
+// allocation holds, aligned to the element (a copy checks the first two itself and takes any alignment).
+bool device_array(const void *p, size_t bytes, size_t align)
+{
+    static const PFN_cuMemGetAddressRange_v3020 range = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const bool ok = cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 3020, cudaEnableDefault, &q) ==
+                            cudaSuccess && q == cudaDriverEntryPointSuccess;
+        return ok ? reinterpret_cast<PFN_cuMemGetAddressRange_v3020>(f) : nullptr;
+    }();
+    cudaPointerAttributes a;
+    int dev = 0;
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    const CUdeviceptr at = (CUdeviceptr)(uintptr_t)p;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == dev && at % align == 0 && range &&
+           range(&base, &size, at) == CUDA_SUCCESS && at - base <= size && bytes <= size - (at - base);
+}
+
 // Device address of a page-locked host array that the device maps (nullptr if p is not one).
 void *mapped_host(const void *p)
 {
@@ -710,7 +757,8 @@ void *mapped_host(const void *p)
 }
 
 // Device addresses of the non-null host arrays p[0..k) if every one is mapped (false otherwise).
-bool all_mapped(const void *const *p, void **d, int k)
+template <typename T>
+bool all_mapped(T *const *p, void **d, int k)
 {
     for (int j = 0; j < k; j++) {
         d[j] = nullptr;
@@ -1101,20 +1149,15 @@ int ann_get_state(ann_ctx *c, double *x, double *y, float *ux, float *uy, float 
     if (!c->have_particles) return fail(c, ANN_ERR_STATE, "no particles");
     const size_t n = (size_t)c->P.n;
     const Bufs &b = c->b;
-    // each field is un-permuted into its own part of the staging buffer (44 bytes per particle of
-    // the 56 it holds), so all copies are in flight before the one synchronisation
     unsigned char *tmp = static_cast<unsigned char *>(c->tmp);
-    struct Part { const void *src; void *dst; int es; } parts[9] = {
-        {b.sx, x, 8}, {b.sy, y, 8}, {b.sux, ux, 4}, {b.suy, uy, 4}, {b.sq11, q11, 4}, {b.sq12, q12, 4}, {b.sdr, drho, 4},
-        {b.sax, ax, 4}, {b.say, ay, 4}};
     const cudaMemcpyKind kind = dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     cudaError_t e = cudaSuccess;
-    const void *dst[9] = {x, y, ux, uy, q11, q12, drho, ax, ay};
+    void *const dst[9] = {x, y, ux, uy, q11, q12, drho, ax, ay};
     void *hd[9];
+    const unsigned nb = (unsigned)((n + 255) / 256);
     if (!dst_is_device && all_mapped(dst, hd, 9)) {
         // page-locked host arrays: one kernel gathers each particle's slot and writes them in
         // particle order over the host link, no staging copy
-        const unsigned nb = (unsigned)((n + 255) / 256);
         int *inv = reinterpret_cast<int *>(tmp);
         k_invert<<<nb, 256, 0, c->stream>>>(b.sid, inv, (int)n);
         k_get_state_mapped<<<nb, 256, 0, c->stream>>>(
@@ -1124,15 +1167,24 @@ int ann_get_state(ann_ctx *c, double *x, double *y, float *ux, float *uy, float 
         if (!e) e = cudaStreamSynchronize(c->stream);
         return e ? cuda_fail(c, e, "ann_get_state") : ANN_OK;
     }
+    // device arrays are written directly (nine copies took 25 of a small state's 45 us); anything else goes
+    // through the staging buffer (44 bytes per particle of the 56 it holds), all copies in flight before
+    // the one synchronisation
+    bool direct = dst_is_device != 0;
+    for (int k = 0; k < 9 && direct; k++)
+        direct = !dst[k] || device_array(dst[k], (k < 2 ? 8 : 4) * n, k < 2 ? 8 : 4);
+    void *out[9];
     size_t off = 0;
-    for (const Part &p : parts) {
-        unsigned char *stage = tmp + off;
-        off += (size_t)p.es * n;
-        if (!p.dst) continue;
-        e = enqueue_unpermute(p.src, b.sid, stage, (int)n, p.es, c->stream);
-        if (!e) e = cudaMemcpyAsync(p.dst, stage, (size_t)p.es * n, kind, c->stream);
-        if (e) break;
+    for (int k = 0; k < 9; k++) {
+        out[k] = !dst[k] || direct ? dst[k] : tmp + off;
+        off += (k < 2 ? 8 : 4) * n;
     }
+    StateDst d{(double *)out[0], (double *)out[1], {}};
+    for (int k = 0; k < 7; k++) d.f[k] = (float *)out[k + 2];
+    k_get_state<<<nb, 256, 0, c->stream>>>(b, (int)n, d);
+    e = cudaGetLastError();
+    for (int k = 0; k < 9 && !e && !direct; k++)
+        if (dst[k]) e = cudaMemcpyAsync(dst[k], out[k], (k < 2 ? 8 : 4) * n, kind, c->stream);
     if (!e) e = cudaStreamSynchronize(c->stream);
     return e ? cuda_fail(c, e, "ann_get_state") : ANN_OK;
 }
