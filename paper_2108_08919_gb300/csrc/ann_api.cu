@@ -854,7 +854,7 @@ int ann_create_with_allocator(const ann_params *p, const ann_allocator *a, ann_c
     c->P = make_dev(*p);
     if (a) c->al = *a;
     cudaError_t e = cudaGetDevice(&c->device);
-    if (!e) e = prepare_kernels();
+    if (!e) e = prepare_kernels(c->P);
     if (!e) e = cudaStreamCreateWithFlags(&c->own, cudaStreamNonBlocking);
     if (!e) e = cudaStreamCreateWithFlags(&c->aux, cudaStreamNonBlocking);
     if (!e) { c->stream = c->own; e = alloc_all(c); }

@@ -157,7 +157,7 @@ __device__ __forceinline__ StateSet state_out(const Bufs &b) { return pick_set(b
 
 // Launch-configuration helpers (defined with the kernels).
 const char *kernel_name(int k);
-cudaError_t prepare_kernels();
+cudaError_t prepare_kernels(const DevParams &P);
 // Launch kernel k (0 <= k < NKERNELS, in step order) of the time step on `s`.  Kernels 1-5 are the
 // re-sort path and kernel 6 its alternative; each also checks the re-sort flag itself.
 cudaError_t launch_kernel(int k, const DevParams &P, const Bufs &b, cudaStream_t s);
