@@ -1734,8 +1734,8 @@ cudaError_t build_ensemble_graph(ann_ensemble *E, int groups)
         E->exec = nullptr;
     }
     // The wider blocks pay where all tiles run at once, here those of `groups` members side by side: 64
-    // members of 128^2 to 512^2 in 16 branches take 2.98 ms a step with 256 threads, 3.07 with 288 (in 64: 2.98, 3.10).  A
-    // particle's sums are the same either way, so members stay bit-identical to solo runs.
+    // members of 128^2 to 512^2 take 2.98 ms a step in 16 branches and in 64 with 256 threads, 3.07 and 3.10
+    // with 288.  A particle's sums are the same either way, so members stay bit-identical to solo runs.
     int64_t tiles = 0;
     for (const ann_ctx *c : E->m) tiles += (int64_t)c->P.tiles * c->P.tiles;
     const int side_by_side = (int)std::min<int64_t>(tiles * groups / (int64_t)E->m.size(), 1 << 30);

@@ -39,8 +39,9 @@ __device__ __forceinline__ bool in_box(double x, long long bitsL)
 // Conversions between FP32 and FP64 in integer arithmetic, bit for bit those of the hardware's
 // instructions.  A conversion runs on the FP64 pipe, at 1/64 of the FP32 rate, and a kernel that walks
 // the particles once is bound by that pipe: the predictor spent 8 of its 14 FP64 operations a particle
-// on conversions (k_predict at 1024^2 particles: 38 us with the instructions, 31 so; k_keys 31 and 21).  Zeros and normal values are done here; FP32 subnormals, overflow, infinity and NaN, which need
-// more than shifts, go to the instruction.
+// on conversions (k_predict at 1024^2 particles: 38 us with the instructions, 31 so; k_keys 31 and 21).
+// Zeros and normal values are done here; FP32 subnormals, overflow, infinity and NaN, which need more than
+// shifts, go to the instruction.
 __device__ __forceinline__ double widen(float f)
 {
     const uint32_t u = __float_as_uint(f);

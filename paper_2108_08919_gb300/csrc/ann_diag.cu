@@ -1,6 +1,6 @@
 // sm_103a kernels of the flow diagnostics of the results section (arXiv 2108.08919, §5): fields on
 // an M x M grid by Shepard interpolation with the method's kernel (Eq. 18), the kinetic-energy
-// spectrum of Eq. 31 by a radix-2 FFT, the vorticity correlation of Eq. 32 along the centre line,
+// spectrum of Eq. 31 by a radix-4 FFT, the vorticity correlation of Eq. 32 along the centre line,
 // topological defects as winding numbers of the gridded Q, the mixing of coloured particles, and
 // unwrapped positions for pathlines.  None of these run inside a step.
 #include "ann_device.cuh"
@@ -11,8 +11,8 @@ namespace ann {
 namespace {
 
 // ------------------------------------------------------------------------------------------------
-// Shepard gridding.  Nodes (ix L/M, iy L/M).  Each node gathers from the particles of the 5 x 5
-// cells around its own cell in the cell order of the last re-sort: a particle has moved far less
+// Shepard gridding.  Nodes (ix L/M, iy L/M).  Each node gathers from the particles of the 3 x 3 or
+// 5 x 5 cells around its own cell in the cell order of the last re-sort: a particle has moved far less
 // than one cell since then (a re-sort comes once anything moves half the 0.02 x 3h skin), so every
 // particle within 3h of the node is in reach, and the sum runs in a fixed order.
 // ------------------------------------------------------------------------------------------------

@@ -772,7 +772,7 @@ __global__ void __launch_bounds__(128) k_gemm_tn(TnArgs a)
 // wgrad: the weight gradients of training,  part[cta] = A^T [B1 | B2 | 1]  over the CTA's row tiles,
 // 128 x (n1 + n2 + 16) FP32 in tensor memory.  A (rows x 128) and B (rows x n) are the row-major
 // activations and adjoints as stored: TMA lands 128-row boxes, whose rows are the K index, so both
-// operands are M/N-major and nothing is transposed (k_gemm_tn below transposes through registers with
+// operands are M/N-major and nothing is transposed (k_gemm_tn above transposes through registers with
 // two-byte shared stores: 27 to 50 us a product at 65,536 rows, 418 us a training step).  The block of
 // ones gives the column sums of A, the bias gradient, in its first column.  Warp 4's first lane loads
 // and issues; warps 0-3 write the CTA's partial sums, which k_wgrad_sum adds in CTA order (so the
