@@ -183,6 +183,20 @@ int lanes_for(int tiles)
     return lanes;
 }
 
+// Whether an ensemble gives a member's particles one thread each, which takes the lanes in turn.  own, side_by_side:
+// particles x lanes of the member, and of all members that run at once.  Lanes on threads of their own shorten
+// a member's chain but cost the GPU more (LP halos staged, LP epilogues, shuffles), so they pay until the threads
+// fill the SMs about eight blocks deep (two rounds of four), and beyond that only where the member's passes
+// are so short that the launches bound them (one block an SM).  Measured, us a step with threads of their own /
+// in turn / one lane, whose sums would not be a solo run's (members side by side): 64^2 x 4 65 / 76 / 71,
+// x 16 148 / 152 / 139; 96^2 x 4 77 / 78 / -, x 6 101 / 88 / -, x 16 230 / 166 / 149; 70^2 x 16 173 / 187 / -; 76^2
+// x 16 176 / 161 / -; 128^2 x 4 77 / 80 / 76, x 16 245 / 192 / 176; 192^2 x 16 353 / 293 / 275.
+bool lanes_in_turn(int64_t own, int64_t side_by_side)
+{
+    const int64_t block_an_sm = 152 * PT_FEW;
+    return own > block_an_sm && side_by_side > 8 * block_an_sm;
+}
+
 // Threads per block of the pair passes.  A cell is at least 3h (1 + skin) wide, 3.98 spacings at h = 1.3 dx,
 // so that a tile holds 250 to 260 particles: with 256 threads about half of the tiles go round their
 // particles twice, the second time for a handful.  Where all tiles run at once (4 to 5 blocks an SM) the
@@ -1736,14 +1750,19 @@ cudaError_t build_ensemble_graph(ann_ensemble *E, int groups)
     // The wider blocks pay where all tiles run at once, here those of `groups` members side by side: 64
     // members of 128^2 to 512^2 take 2.98 ms a step in 16 branches and in 64 with 256 threads, 3.07 and 3.10
     // with 288.  A particle's sums are the same either way, so members stay bit-identical to solo runs.
-    int64_t tiles = 0;
-    for (const ann_ctx *c : E->m) tiles += (int64_t)c->P.tiles * c->P.tiles;
-    const int side_by_side = (int)std::min<int64_t>(tiles * groups / (int64_t)E->m.size(), 1 << 30);
+    int64_t tiles = 0, threads = 0;
+    for (const ann_ctx *c : E->m) {
+        tiles += (int64_t)c->P.tiles * c->P.tiles;
+        threads += (int64_t)c->P.n * c->P.lanes;
+    }
+    auto side_by_side = [&](int64_t all, int64_t own) { return std::max(all * groups / (int64_t)E->m.size(), own); };
     std::vector<DevParams> P;
     cudaError_t e = cudaSuccess;
     for (const ann_ctx *c : E->m) {
+        const int64_t own_tiles = (int64_t)c->P.tiles * c->P.tiles, own = (int64_t)c->P.n * c->P.lanes;
         P.push_back(c->P);
-        P.back().threads = threads_for(std::max(side_by_side, c->P.tiles * c->P.tiles));
+        P.back().threads = threads_for((int)std::min<int64_t>(side_by_side(tiles, own_tiles), 1 << 30));
+        P.back().in_turn = lanes_in_turn(own, side_by_side(threads, own));
         if (!e) e = prepare_kernels(P.back());
     }
     if (e) return e;

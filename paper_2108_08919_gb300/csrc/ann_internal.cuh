@@ -52,6 +52,7 @@ enum : uint32_t {
 struct DevParams {
     int n, nc, ncell, tiles;
     int lanes;             // lanes per particle of passes A to D (1, 2, 4 or 8), by the tile count
+    int in_turn;           // one thread takes its particle's lanes in turn (see lanes_in_turn)
     int threads;           // threads per block of the pair passes (PT or PT_FEW), by the tile count
     int apd, conservative, qnew, record, elastic;
     double L, cell, inv_cell, R2, dt_d, half_dt_d;

@@ -71,18 +71,18 @@ struct Tile {
 
 __device__ __forceinline__ bool first_thread() { return (blockIdx.x | blockIdx.y | threadIdx.x) == 0; }
 
-// Set up by the block's first warp; blocks are a grid of tiles (x, y), LP blocks per tile along x (see
+// Set up by the block's first warp; blocks are a grid of tiles (x, y), LP blocks per tile along x or, in turn, one (see
 // "Lanes per particle" below).  Everything a thread does per tile or per slot counts: with a search
 // loop and divisions per slot, and a prefix by one thread, set-up and staging were a third of the
 // instructions of a pass; now they are 200 of 2,150 to 2,900 per warp (512^2: A 27.7 -> 25.6 us, D 35.8 ->
 // 34.7).  False: an error has been raised, here (the halo does not fit) or before -- decided once for the
 // whole block, since another block may raise one at any time.
-template <int LP = 1>
+template <int LP = 1, bool TURN = false>
 __device__ __forceinline__ bool tile_begin(const DevParams &P, const Bufs &b, TileShared &ts, Tile &T)
 {
     const int t = threadIdx.x;
     if (t < 32) {
-        const int cx0 = (int)(blockIdx.x / LP) * TILE, cy0 = (int)blockIdx.y * TILE;
+        const int cx0 = (int)(blockIdx.x / (TURN ? 1 : LP)) * TILE, cy0 = (int)blockIdx.y * TILE;
         const int wx = min(TILE, P.nc - cx0), wy = min(TILE, P.nc - cy0);
         const bool stop = stopped(b);
         int first[2], cnt[2];   // halo cells t and t + 32
@@ -609,34 +609,9 @@ __global__ void __launch_bounds__(T) k_pass_a_resort(DevParams P, Bufs b)
 // next PF words in flight while the current ones are processed: fn(byte offset of the slot,
 // candidate index, bit), bit = the entry's neighbour bit (nonzero iff the candidate is a neighbour).
 // Word m (candidates 4m .. 4m + 3) is loaded only when 4m < c.
-// With LP > 1 lanes per particle, lane l visits the words l, l + LP, ...
-template <int PF, int LP = 1, typename Fn>
+template <int PF, typename Fn>
 __device__ __forceinline__ void for_each_slot(const uint2 *list, int n, int gi, int c, Fn &&fn)
 {
-    if constexpr (LP > 1) {
-        const int l = threadIdx.x & (LP - 1);
-        const uint2 *p = list + (size_t)l * n + gi;
-        uint2 nxt = 4 * l < c ? __ldg(p) : make_uint2(0u, 0u);
-        for (int k = 4 * l; k < c; k += 4 * LP) {
-            const uint2 w = nxt;
-            p += (size_t)LP * n;
-            if (k + 4 * LP < c) nxt = __ldg(p);
-            if (k + 3 < c) {
-                fn((int)(w.x & SLOT_OFF_MASK), k, w.x & 1u);
-                fn((int)((w.x >> 16) & SLOT_OFF_MASK), k + 1, w.x & 0x10000u);
-                fn((int)(w.y & SLOT_OFF_MASK), k + 2, w.y & 1u);
-                fn((int)((w.y >> 16) & SLOT_OFF_MASK), k + 3, w.y & 0x10000u);
-            } else {
-                const unsigned long long w64 = ((unsigned long long)w.y << 32) | w.x;
-                for (int t = 0; k + t < c; t++) {
-                    const unsigned e = (unsigned)(w64 >> (16 * t));
-                    fn((int)(e & SLOT_OFF_MASK), k + t, e & 1u);
-                }
-            }
-        }
-        return;
-    }
-
     static_assert(PF >= 1 && PF <= 3, "prefetch distance");
     const uint2 *p = list + gi;
     uint2 r[PF + 1];   // r[0]: the current word, r[m]: word k/4 + m
@@ -664,20 +639,23 @@ __device__ __forceinline__ void for_each_slot(const uint2 *list, int n, int gi, 
 
 // Candidates of particle gi.  Beyond the support the clamped kernel gives W = F = 0 exactly, and
 // adding +0 or -0 leaves an FP32 sum unchanged, so sums over candidates equal sums over neighbours.
-template <int PF, int LP = 1, typename Fn>
+template <int PF, typename Fn>
 __device__ __forceinline__ void for_each_candidate(const DevParams &P, const Bufs &b, int gi, Fn &&fn)
 {
-    for_each_slot<PF, LP>(b.vnbr, P.n, gi, b.vcnt[gi], fn);
+    for_each_slot<PF>(b.vnbr, P.n, gi, b.vcnt[gi], fn);
 }
 
 // Lanes per particle (P.lanes: 1, 2, 4 or 8, the template argument LP of the passes).  A box of few
 // tiles leaves the GPU idle with one block per tile and one thread per particle: 64^2 has 16 tiles for
 // 152 SMs, and a thread's walk of 46 candidates is most of a pass.  There LP blocks share a tile (each
 // stages the whole halo and takes its share of the particles, T / LP at a time) and LP lanes a particle's candidate words.
-template <int LP, int T>
+// An ensemble whose members fill the GPU together gets one block per tile and one thread per particle all the same
+// (P.in_turn, see lanes_in_turn), and that thread takes the lanes one after the other and joins their sums in the
+// lanes' order: the same instructions in the same order, so a member ends with the bits of a run on its own.
+template <int LP, int T, bool TURN>
 __device__ __forceinline__ int first_particle()
 {
-    return (int)((blockIdx.x % LP) * T + threadIdx.x) / LP;
+    return TURN ? (int)threadIdx.x : (int)((blockIdx.x % LP) * T + threadIdx.x) / LP;
 }
 
 // The lanes' sums; every lane of the particle gets the total (a no-op for one lane).
@@ -707,11 +685,98 @@ __device__ __forceinline__ int lane_sum(int v)
     }
     return v;
 }
+// Joins the sums of a thread that takes the lanes in turn, in the order of lane_sum's tree: a lane's sums are added
+// to those of the lanes before it that are complete, so that at most log2 LP sets wait (in local memory).
+template <int LP, bool TURN, int N>
+struct LaneTree {
+    float s[3][N];   // LP <= 8
+    __device__ __forceinline__ static void add(const float *t, int &j, float &a) { a = t[j++] + a; }
+    __device__ __forceinline__ static void add(const float *t, int &j, float2 &a)
+    {
+        a = f2(t[j] + a.x, t[j + 1] + a.y);
+        j += 2;
+    }
+    __device__ __forceinline__ static void put(float *t, int &j, float a) { t[j++] = a; }
+    __device__ __forceinline__ static void put(float *t, int &j, float2 a)
+    {
+        t[j++] = a.x;
+        t[j++] = a.y;
+    }
+    template <typename... A>
+    __device__ __forceinline__ void join(int l, A &...a)
+    {
+        int k = 0;
+        for (; (l >> k) & 1; k++) {
+            int j = 0;
+            (add(s[k], j, a), ...);
+        }
+        if (l + 1 < LP) {
+            int j = 0;
+            (put(s[k], j, a), ...);
+        }
+    }
+};
+template <int LP, int N>
+struct LaneTree<LP, false, N> {
+    template <typename... A>
+    __device__ __forceinline__ void join(int, A &...)
+    {
+    }
+};
+
+// A thread's lanes of its particle: l = first() .. last() in steps of one (its own lane, or all of them in turn).
+// Lane l visits the list words l, l + LP, ...; the next lane's first word is in flight while one is walked.
+template <int LP, bool TURN>
+struct LaneWords {
+    const uint2 *p;
+    int n, c;
+    uint2 head;
+    __device__ __forceinline__ LaneWords(const DevParams &P, const Bufs &b, int gi)
+        : p(b.vnbr + gi), n(P.n), c(b.vcnt[gi])
+    {
+        if (LP > 1) head = 4 * first() < c ? __ldg(p + (size_t)first() * n) : make_uint2(0u, 0u);
+    }
+    __device__ __forceinline__ int first() const { return LP == 1 || TURN ? 0 : (int)(threadIdx.x & (LP - 1)); }
+    __device__ __forceinline__ int last() const { return TURN ? LP - 1 : first(); }
+    template <int PF, typename Fn>
+    __device__ __forceinline__ void walk(int l, Fn &&fn)
+    {
+        if constexpr (LP == 1) {
+            for_each_slot<PF>(p, n, 0, c, fn);
+        } else {
+            const uint2 *q = p + (size_t)l * n;
+            uint2 nxt = head;
+            if (l < last() && 4 * (l + 1) < c) head = __ldg(q + n);
+            for (int k = 4 * l; k < c; k += 4 * LP) {
+                const uint2 w = nxt;
+                q += (size_t)LP * n;
+                if (k + 4 * LP < c) nxt = __ldg(q);
+                if (k + 3 < c) {
+                    fn((int)(w.x & SLOT_OFF_MASK), k, w.x & 1u);
+                    fn((int)((w.x >> 16) & SLOT_OFF_MASK), k + 1, w.x & 0x10000u);
+                    fn((int)(w.y & SLOT_OFF_MASK), k + 2, w.y & 1u);
+                    fn((int)((w.y >> 16) & SLOT_OFF_MASK), k + 3, w.y & 0x10000u);
+                } else {
+                    const unsigned long long w64 = ((unsigned long long)w.y << 32) | w.x;
+                    for (int t = 0; k + t < c; t++) {
+                        const unsigned e = (unsigned)(w64 >> (16 * t));
+                        fn((int)(e & SLOT_OFF_MASK), k + t, e & 1u);
+                    }
+                }
+            }
+        }
+    }
+};
+
+// a b + c d.  Left to the compiler, which of the two products the addition takes in may differ between instances of a
+// kernel, and with it the last bit.
+__device__ __forceinline__ float dot2(float a, float b, float c, float d) { return fmaf(a, b, __fmul_rn(c, d)); }
+
 // Whether this lane writes the particle's results.
-template <int LP>
+template <int LP, bool TURN>
 __device__ __forceinline__ bool writes()
 {
-    return LP == 1 || (threadIdx.x & (LP - 1)) == 0;
+    return LP == 1 || TURN || (threadIdx.x & (LP - 1)) == 0;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -721,7 +786,7 @@ __device__ __forceinline__ bool writes()
 
 constexpr int SMEM_AF = HCAP * (16 + 4);
 
-template <int LP, int T>
+template <int LP, int T, bool TURN>
 __global__ void BOUNDS_A k_pass_a_filter(DevParams P, Bufs b)
 {
     if (resorting(b)) return;
@@ -730,14 +795,14 @@ __global__ void BOUNDS_A k_pass_a_filter(DevParams P, Bufs b)
     float4 *pos = reinterpret_cast<float4 *>(dsm);
     int *sg = reinterpret_cast<int *>(pos + HCAP);
     Tile tile;
-    if (!tile_begin<LP>(P, b, ts, tile)) return;
+    if (!tile_begin<LP, TURN>(P, b, ts, tile)) return;
     for (int t = threadIdx.x; t < tile.H; t += T) {
         SlotInfo s = slot_info(P, b, ts, t);
         pos[t] = s.e;
         sg[t] = s.g;
     }
     __syncthreads();
-    for (int q = first_particle<LP, T>(); q < tile.Ni; q += T) {
+    for (int q = first_particle<LP, T, TURN>(); q < tile.Ni; q += T) {
         int si = inner_slot(ts, q);
         int gi = sg[si];
         float4 pi = pos[si];
@@ -748,6 +813,12 @@ __global__ void BOUNDS_A k_pass_a_filter(DevParams P, Bufs b)
         // in FP64 by a second walk.  A word is stored only when a bit changed (a pair crossed 3h).
         int nn = 0;
         bool band = false;
+        // the lanes' words as in LaneWords, by plain loads: this kernel writes the words
+        const int first = LP == 1 || TURN ? 0 : (int)(threadIdx.x & (LP - 1));
+        const int last = TURN ? LP - 1 : first;
+        const size_t stride = (size_t)LP * P.n;
+        uint2 head = 4 * first < c ? b.vnbr[(size_t)first * P.n + gi] : make_uint2(0u, 0u);
+        LaneTree<LP, TURN, 1> tree;
         auto test = [&](uint32_t e) {
             const uint32_t o = e & SLOT_OFF_MASK;
             float r2 = len2(pair_d(pi, slot_at(pos, (int)o)));
@@ -757,45 +828,55 @@ __global__ void BOUNDS_A k_pass_a_filter(DevParams P, Bufs b)
             nn += (int)in;
             return o | in;
         };
-        const int l = threadIdx.x & (LP - 1);   // this lane's words: l, l + LP, ...
-        const size_t stride = (size_t)LP * P.n;
-        uint2 *p = b.vnbr + (size_t)l * P.n + gi;
-        uint2 nxt = 4 * l < c ? *p : make_uint2(0u, 0u);   // plain loads: this kernel writes the words
-        int k = 4 * l;
-        for (; k + 3 < c; k += 4 * LP, p += stride) {
-            const uint2 w = nxt;
-            if (k + 4 * LP < c) nxt = p[stride];   // the next word, in flight while this one is done
-            const uint32_t e0 = test(w.x & 0xffffu), e1 = test(w.x >> 16), e2 = test(w.y & 0xffffu),
-                           e3 = test(w.y >> 16);
-            const uint2 v = make_uint2(e0 | (e1 << 16), e2 | (e3 << 16));
-            if (v.x != w.x || v.y != w.y) *p = v;
-        }
-        if (k < c) {   // the last word, 1 to 3 candidates (the rest of it is zero)
-            const uint2 w = nxt;
-            uint32_t e[4] = {w.x & 0xffffu, w.x >> 16, w.y & 0xffffu, w.y >> 16};
-            for (int t = 0; t < c - k; t++) e[t] = test(e[t]);
-            const uint2 v = make_uint2(e[0] | (e[1] << 16), e[2] | (e[3] << 16));
-            if (v.x != w.x || v.y != w.y) *p = v;
-        }
-        if (band) {   // the band's candidates, decided in FP64 (the FP32 test left their bit 0)
-            uint2 *q = b.vnbr + (size_t)l * P.n + gi;
-            for (int k0 = 4 * l; k0 < c; k0 += 4 * LP, q += stride) {
-                uint2 w = *q;
-                uint32_t e[4] = {w.x & 0xffffu, w.x >> 16, w.y & 0xffffu, w.y >> 16};
-                for (int t = 0; t < 4 && k0 + t < c; t++) {
-                    const int o = (int)(e[t] & SLOT_OFF_MASK);
-                    float r2 = len2(pair_d(pi, slot_at(pos, o)));
-                    if (r2 >= P.R2lo && in_support(r2, P, b, gi, slot_at(sg, o))) {
-                        e[t] |= 1u;
-                        nn++;
-                    }
-                }
-                *q = make_uint2(e[0] | (e[1] << 16), e[2] | (e[3] << 16));
+#pragma unroll 1
+        for (int l = first; l <= last; l++) {
+            if (LP > 1) {
+                sw = 0.f;
+                band = false;
             }
+            uint2 *p = b.vnbr + (size_t)l * P.n + gi;
+            uint2 nxt = head;
+            if (l < last && 4 * (l + 1) < c) head = p[P.n];
+            int k = 4 * l;
+            for (; k + 3 < c; k += 4 * LP, p += stride) {
+                const uint2 w = nxt;
+                if (k + 4 * LP < c) nxt = p[stride];   // the next word, in flight while this one is done
+                const uint32_t e0 = test(w.x & 0xffffu), e1 = test(w.x >> 16), e2 = test(w.y & 0xffffu),
+                               e3 = test(w.y >> 16);
+                const uint2 v = make_uint2(e0 | (e1 << 16), e2 | (e3 << 16));
+                if (v.x != w.x || v.y != w.y) *p = v;
+            }
+            if (k < c) {   // the last word, 1 to 3 candidates (the rest of it is zero)
+                const uint2 w = nxt;
+                uint32_t e[4] = {w.x & 0xffffu, w.x >> 16, w.y & 0xffffu, w.y >> 16};
+                for (int t = 0; t < c - k; t++) e[t] = test(e[t]);
+                const uint2 v = make_uint2(e[0] | (e[1] << 16), e[2] | (e[3] << 16));
+                if (v.x != w.x || v.y != w.y) *p = v;
+            }
+            if (band) {   // the band's candidates, decided in FP64 (the FP32 test left their bit 0)
+                uint2 *q = b.vnbr + (size_t)l * P.n + gi;
+                for (int k0 = 4 * l; k0 < c; k0 += 4 * LP, q += stride) {
+                    uint2 w = *q;
+                    uint32_t e[4] = {w.x & 0xffffu, w.x >> 16, w.y & 0xffffu, w.y >> 16};
+                    for (int t = 0; t < 4 && k0 + t < c; t++) {
+                        const int o = (int)(e[t] & SLOT_OFF_MASK);
+                        float r2 = len2(pair_d(pi, slot_at(pos, o)));
+                        if (r2 >= P.R2lo && in_support(r2, P, b, gi, slot_at(sg, o))) {
+                            e[t] |= 1u;
+                            nn++;
+                        }
+                    }
+                    *q = make_uint2(e[0] | (e[1] << 16), e[2] | (e[3] << 16));
+                }
+            }
+            tree.join(l, sw);
         }
-        nn = lane_sum<LP>(nn);
-        if (LP > 1) sw = P.W0 + lane_sum<LP>(sw);
-        if (!writes<LP>()) continue;
+        if (!TURN) {
+            nn = lane_sum<LP>(nn);
+            sw = lane_sum<LP>(sw);
+        }
+        if (LP > 1) sw = P.W0 + sw;
+        if (!writes<LP, TURN>()) continue;
         b.nnbr[gi] = nn;
         b.sumW[gi] = sw;
         b.V[gi] = 1.0f / sw;
@@ -810,7 +891,7 @@ __global__ void BOUNDS_A k_pass_a_filter(DevParams P, Bufs b)
 
 constexpr int SMEM_B = HCAP * (16 + 16 + 4 + 4);
 
-template <bool QOLD, int LP, int T>
+template <bool QOLD, int LP, int T, bool TURN>
 __global__ void BOUNDS_B k_pass_b(DevParams P, Bufs b)
 {
     __shared__ TileShared ts;
@@ -820,7 +901,7 @@ __global__ void BOUNDS_B k_pass_b(DevParams P, Bufs b)
     float *sv = reinterpret_cast<float *>(sb + HCAP); // V
     int *sg = reinterpret_cast<int *>(sv + HCAP);
     Tile tile;
-    if (!tile_begin<LP>(P, b, ts, tile)) return;
+    if (!tile_begin<LP, TURN>(P, b, ts, tile)) return;
     if (first_thread()) *b.rebuild = 0u;   // both pass A kernels have run
     for (int t = threadIdx.x; t < tile.H; t += T) {
         SlotInfo s = slot_info(P, b, ts, t);
@@ -830,7 +911,7 @@ __global__ void BOUNDS_B k_pass_b(DevParams P, Bufs b)
         sg[t] = s.g;
     }
     __syncthreads();
-    for (int q = first_particle<LP, T>(); q < tile.Ni; q += T) {
+    for (int q = first_particle<LP, T, TURN>(); q < tile.Ni; q += T) {
         int si = inner_slot(ts, q);
         int gi = sg[si];
         float4 pi = sp[si], bi = sb[si];
@@ -842,30 +923,41 @@ __global__ void BOUNDS_B k_pass_b(DevParams P, Bufs b)
         float a22 = 0.f;
         float di = b.mdr[gi];   // loaded ahead of the neighbour loop
         const float2 ui = f2(bi.x, bi.y), qi = f2(bi.z, bi.w);
-        for_each_candidate<ANN_PF_B, LP>(P, b, gi, [&](int o, int, unsigned) {
-            float4 bj = slot_at(sb, o);
-            float2 d = pair_d(pi, slot_at(sp, o));
-            KernelPowers kp = kernel_powers<true>(len2(d), P);
-            float F = kernel_f_of(kp, P);
-            float2 g = mul2(bc(slot_at(sv, o) * F), d);  // V_j grad_i W = (gx, gy)
-            float2 mx = mul2(bc(g.x), d);                 // (mxx, mxy)
-            float myy = g.y * d.y;
-            a1 = sub2(a1, mx);
-            a22 -= myy;
-            float2 du = sub2(f2(bj.x, bj.y), ui);         // u_j - u_i
-            l0 = fma2(bc(du.x), g, l0);
-            l1 = fma2(bc(du.y), g, l1);
-            float2 dq = sub2(f2(bj.z, bj.w), qi);         // Q_j - Q_i per component
-            float2 e = mul2(dq, bc(-(kp.rinv * kp.rinv)));
-            rxx = fma2(e, bc(mx.x), rxx);
-            rxy = fma2(e, bc(mx.y), rxy);
-            ryy = fma2(e, bc(myy), ryy);
-            if (QOLD) {
-                gq1 = fma2(bc(dq.x), g, gq1);
-                gq2 = fma2(bc(dq.y), g, gq2);
+        LaneWords<LP, TURN> words(P, b, gi);
+        LaneTree<LP, TURN, QOLD ? 17 : 13> tree;
+#pragma unroll 1
+        for (int l = words.first(); l <= words.last(); l++) {
+            if (LP > 1) {
+                a1 = l0 = l1 = rxx = rxy = ryy = gq1 = gq2 = f2(0.f, 0.f);
+                a22 = 0.f;
             }
-        });
-        if (LP > 1) {
+            words.template walk<ANN_PF_B>(l, [&](int o, int, unsigned) {
+                float4 bj = slot_at(sb, o);
+                float2 d = pair_d(pi, slot_at(sp, o));
+                KernelPowers kp = kernel_powers<true>(len2(d), P);
+                float F = kernel_f_of(kp, P);
+                float2 g = mul2(bc(slot_at(sv, o) * F), d);  // V_j grad_i W = (gx, gy)
+                float2 mx = mul2(bc(g.x), d);                 // (mxx, mxy)
+                float myy = g.y * d.y;
+                a1 = sub2(a1, mx);
+                a22 -= myy;
+                float2 du = sub2(f2(bj.x, bj.y), ui);         // u_j - u_i
+                l0 = fma2(bc(du.x), g, l0);
+                l1 = fma2(bc(du.y), g, l1);
+                float2 dq = sub2(f2(bj.z, bj.w), qi);         // Q_j - Q_i per component
+                float2 e = mul2(dq, bc(-(kp.rinv * kp.rinv)));
+                rxx = fma2(e, bc(mx.x), rxx);
+                rxy = fma2(e, bc(mx.y), rxy);
+                ryy = fma2(e, bc(myy), ryy);
+                if (QOLD) {
+                    gq1 = fma2(bc(dq.x), g, gq1);
+                    gq2 = fma2(bc(dq.y), g, gq2);
+                }
+            });
+            if (QOLD) tree.join(l, a1, a22, l0, l1, rxx, rxy, ryy, gq1, gq2);
+            else tree.join(l, a1, a22, l0, l1, rxx, rxy, ryy);
+        }
+        if (LP > 1 && !TURN) {
             a1 = lane_sum<LP>(a1);
             a22 = lane_sum<LP>(a22);
             l0 = lane_sum<LP>(l0);
@@ -877,7 +969,7 @@ __global__ void BOUNDS_B k_pass_b(DevParams P, Bufs b)
                 gq1 = lane_sum<LP>(gq1);
                 gq2 = lane_sum<LP>(gq2);
             }
-            if (!writes<LP>()) continue;
+            if (!writes<LP, TURN>()) continue;
         }
         float a11 = a1.x, a12 = a1.y;
         float l00 = l0.x, l01 = l0.y, l10 = l1.x, l11 = l1.y;
@@ -929,10 +1021,10 @@ __global__ void BOUNDS_B k_pass_b(DevParams P, Bufs b)
         b.bk[gi] = make_float4(B11, B12, B22, kr);
         b.cr[gi] = make_float4(sv[si], di + P.half_dt * kr, q1n, q2n);   // pass C's staged record
         if (QOLD) {   // div Q^n for pass D (pass C then leaves the divergence part of cq alone)
-            float q1x = g1x * B11 + g1y * B12, q1y = g1x * B12 + g1y * B22;
-            float q2x = g2x * B11 + g2y * B12, q2y = g2x * B12 + g2y * B22;
+            float q1x = dot2(g1x, B11, g1y, B12), q1y = dot2(g1x, B12, g1y, B22);
+            float q2x = dot2(g2x, B11, g2y, B12), q2y = dot2(g2x, B12, g2y, B22);
             float2 *dq = reinterpret_cast<float2 *>(b.cq + gi);
-            *dq = make_float2(q1x + q2y, q2x - q1y);
+            *dq = make_float2(__fadd_rn(q1x, q2y), __fsub_rn(q2x, q1y));
         }
         if (P.record) {
             b.rec_gu[4 * gi + 0] = D00;
@@ -954,7 +1046,7 @@ __global__ void BOUNDS_B k_pass_b(DevParams P, Bufs b)
 // the elastic stress tile exists only in the instantiations that read it
 constexpr int smem_c(bool el) { return HCAP * (16 + 16 + (el ? 16 : 0) + 4); }
 
-template <bool QNEW, bool EL, int LP, int T>
+template <bool QNEW, bool EL, int LP, int T, bool TURN>
 __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
 {
     __shared__ TileShared ts;
@@ -964,7 +1056,7 @@ __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
     float4 *se = sb + HCAP;                            // elastic stress (11, 12, 22, -)
     int *sg = reinterpret_cast<int *>(se + (EL ? HCAP : 0));
     Tile tile;
-    if (!tile_begin<LP>(P, b, ts, tile)) return;
+    if (!tile_begin<LP, TURN>(P, b, ts, tile)) return;
     const StateSet out = state_out(b);   // Q^{n+1} (pass B)
     for (int t = threadIdx.x; t < tile.H; t += T) {
         SlotInfo s = slot_info(P, b, ts, t);
@@ -981,7 +1073,7 @@ __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
     if (P.dt_check && first_thread() &&
         (P.dt > P.dt_static || P.dt * (c0 + umax) * P.inv_h > 0.25f))
         atomicOr(b.err, EB_CFL);
-    for (int q = first_particle<LP, T>(); q < tile.Ni; q += T) {
+    for (int q = first_particle<LP, T, TURN>(); q < tile.Ni; q += T) {
         int si = inner_slot(ts, q);
         int gi = sg[si];
         float4 pi = sp[si], bi = sb[si];
@@ -999,28 +1091,41 @@ __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
         float2 gq1 = f2(0.f, 0.f), gq2 = f2(0.f, 0.f), ge1 = f2(0.f, 0.f), ge2 = f2(0.f, 0.f),
                ge3 = f2(0.f, 0.f);
         const float2 qi = f2(bi.z, bi.w);
-        for_each_candidate<ANN_PF_C, LP>(P, b, gi, [&](int o, int, unsigned) {
-            float4 bj = slot_at(sb, o);
-            float2 d = pair_d(pi, slot_at(sp, o));
-            KernelPowers kp = kernel_powers<true>(len2(d), P);
-            float Wv = kernel_w_of(kp, P);
-            shep += (bi.y - bj.y) * Wv;
-            if (QNEW || EL) {
-                float2 g = mul2(bc(bj.x * kernel_f_of(kp, P)), d);
-                if (QNEW) {
-                    float2 dq = sub2(f2(bj.z, bj.w), qi);
-                    gq1 = fma2(bc(dq.x), g, gq1);
-                    gq2 = fma2(bc(dq.y), g, gq2);
-                }
-                if (EL) {
-                    float4 ej = slot_at(se, o);
-                    ge1 = fma2(bc(ej.x - ei.x), g, ge1);
-                    ge2 = fma2(bc(ej.y - ei.y), g, ge2);
-                    ge3 = fma2(bc(ej.z - ei.z), g, ge3);
-                }
+        LaneWords<LP, TURN> words(P, b, gi);
+        LaneTree<LP, TURN, 1 + (QNEW ? 4 : 0) + (EL ? 6 : 0)> tree;
+#pragma unroll 1
+        for (int l = words.first(); l <= words.last(); l++) {
+            if (LP > 1) {
+                shep = 0.f;
+                gq1 = gq2 = ge1 = ge2 = ge3 = f2(0.f, 0.f);
             }
-        });
-        if (LP > 1) {
+            words.template walk<ANN_PF_C>(l, [&](int o, int, unsigned) {
+                float4 bj = slot_at(sb, o);
+                float2 d = pair_d(pi, slot_at(sp, o));
+                KernelPowers kp = kernel_powers<true>(len2(d), P);
+                float Wv = kernel_w_of(kp, P);
+                shep += (bi.y - bj.y) * Wv;
+                if (QNEW || EL) {
+                    float2 g = mul2(bc(bj.x * kernel_f_of(kp, P)), d);
+                    if (QNEW) {
+                        float2 dq = sub2(f2(bj.z, bj.w), qi);
+                        gq1 = fma2(bc(dq.x), g, gq1);
+                        gq2 = fma2(bc(dq.y), g, gq2);
+                    }
+                    if (EL) {
+                        float4 ej = slot_at(se, o);
+                        ge1 = fma2(bc(ej.x - ei.x), g, ge1);
+                        ge2 = fma2(bc(ej.y - ei.y), g, ge2);
+                        ge3 = fma2(bc(ej.z - ei.z), g, ge3);
+                    }
+                }
+            });
+            if (QNEW && EL) tree.join(l, shep, gq1, gq2, ge1, ge2, ge3);
+            else if (QNEW) tree.join(l, shep, gq1, gq2);
+            else if (EL) tree.join(l, shep, ge1, ge2, ge3);
+            else tree.join(l, shep);
+        }
+        if (LP > 1 && !TURN) {
             shep = lane_sum<LP>(shep);
             if (QNEW) {
                 gq1 = lane_sum<LP>(gq1);
@@ -1031,7 +1136,7 @@ __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
                 ge2 = lane_sum<LP>(ge2);
                 ge3 = lane_sum<LP>(ge3);
             }
-            if (!writes<LP>()) continue;
+            if (!writes<LP, TURN>()) continue;
         }
         float g1x = gq1.x, g1y = gq1.y, g2x = gq2.x, g2y = gq2.y;
         float e1x = ge1.x, e1y = ge1.y, e2x = ge2.x, e2y = ge2.y, e3x = ge3.x, e3y = ge3.y;
@@ -1045,19 +1150,19 @@ __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
             b.rd[gi] = make_float4(bi.x, pg * irho * irho, u.x, u.y);
         }
         if (QNEW) {
-            float q1x = g1x * B11 + g1y * B12, q1y = g1x * B12 + g1y * B22;
-            float q2x = g2x * B11 + g2y * B12, q2y = g2x * B12 + g2y * B22;
-            b.cq[gi] = make_float4(q1x + q2y, q2x - q1y, dhat, swi);
+            float q1x = dot2(g1x, B11, g1y, B12), q1y = dot2(g1x, B12, g1y, B22);
+            float q2x = dot2(g2x, B11, g2y, B12), q2y = dot2(g2x, B12, g2y, B22);
+            b.cq[gi] = make_float4(__fadd_rn(q1x, q2y), __fsub_rn(q2x, q1y), dhat, swi);
         } else {   // div Q^n came from pass B
             float2 *hs = reinterpret_cast<float2 *>(b.cq + gi) + 1;
             *hs = make_float2(dhat, swi);
         }
         if (EL) {   // div Pi = (d_x Pi11 + d_y Pi12, d_x Pi12 + d_y Pi22), corrected gradients
-            float p11x = e1x * B11 + e1y * B12;
-            float p12x = e2x * B11 + e2y * B12, p12y = e2x * B12 + e2y * B22;
-            float p22y = e3x * B12 + e3y * B22;
-            b.delx[gi] = p11x + p12y;
-            b.dely[gi] = p12x + p22y;
+            float p11x = dot2(e1x, B11, e1y, B12);
+            float p12x = dot2(e2x, B11, e2y, B12), p12y = dot2(e2x, B12, e2y, B22);
+            float p22y = dot2(e3x, B12, e3y, B22);
+            b.delx[gi] = __fadd_rn(p11x, p12y);
+            b.dely[gi] = __fadd_rn(p12x, p22y);
         }
     }
 }
@@ -1069,7 +1174,7 @@ __global__ void BOUNDS_C k_pass_c(DevParams P, Bufs b)
 // (the (q11, q12)/rho^2 tile exists in the conservative mode only, Pi/rho^2 with the elastic stress)
 constexpr int smem_d(bool cons, bool el) { return HCAP * (16 + 16 + (cons ? 8 : 0) + (cons && el ? 16 : 0) + 4); }
 
-template <bool CONS, bool EL, int LP, int T>
+template <bool CONS, bool EL, int LP, int T, bool TURN>
 __global__ void BOUNDS_D k_pass_d(DevParams P, Bufs b)
 {
     __shared__ TileShared ts;
@@ -1082,7 +1187,7 @@ __global__ void BOUNDS_D k_pass_d(DevParams P, Bufs b)
     // the step's output set: Q^{n+1} (pass B) in, the new state out; k_commit of the next step (or
     // the host) commits it if no error has been raised by then
     Tile tile;
-    if (!tile_begin<LP>(P, b, ts, tile)) return;
+    if (!tile_begin<LP, TURN>(P, b, ts, tile)) return;
     if (first_thread()) b.ctl[CTL_PENDING] = 1u;
     const StateSet out = state_out(b);
     for (int t = threadIdx.x; t < tile.H; t += T) {
@@ -1109,7 +1214,7 @@ __global__ void BOUNDS_D k_pass_d(DevParams P, Bufs b)
     }
     __syncthreads();
     if (first_thread()) *b.maxu = 0u;   // pass C has consumed it
-    for (int q = first_particle<LP, T>(); q < tile.Ni; q += T) {
+    for (int q = first_particle<LP, T, TURN>(); q < tile.Ni; q += T) {
         int si = inner_slot(ts, q);
         int gi = sg[si];
         float4 pi = sp[si], bi = sb[si];
@@ -1130,48 +1235,58 @@ __global__ void BOUNDS_D k_pass_d(DevParams P, Bufs b)
         const float2 ui = f2(bi.z, bi.w);
         float2 w = f2(0.f, 0.f), su = f2(0.f, 0.f), sd = f2(0.f, 0.f);
         float sr = 0.f;
-        for_each_candidate<ANN_PF_D, LP>(P, b, gi, [&](int o, int, unsigned in) {
-            float4 bj = slot_at(sb, o);
-            float2 d = pair_d(pi, slot_at(sp, o));
-            float r2 = len2(d);
-            KernelPowers kp = kernel_powers<true>(r2, P);
-            float Wv = kernel_w_of(kp, P), F = kernel_f_of(kp, P);
-            float2 du = sub2(ui, f2(bj.z, bj.w));   // u_i - u_j
-            float ud = fmaf(du.x, d.x, du.y * d.y);
-            float rinv2 = kp.rinv * kp.rinv;
-            if (CONS) {
-                float2 cj = slot_at(sc, o);
-                float2 g = mul2(bc(F), d);
-                float visc = k8 * bj.y * ud * rinv2;
-                w = fma2(bc(visc - (bi.x + bj.x)), g, w);
-                float2 qs = add2(ci, cj);   // (Q11_i/rho_i^2 + Q11_j/rho_j^2, same for Q12)
-                // Q.g = (qa gx + qb gy, qb gx - qa gy)
-                float2 act = fma2(qs, bc(g.x), mul2(f2(qs.y, -qs.x), bc(g.y)));
-                w = fma2(bc(-P.zeta), act, w);
-                if (EL) {   // + sum_j m (Pi_i/rho_i^2 + Pi_j/rho_j^2) . grad_i W
-                    float4 ecj = slot_at(se, o);
-                    float2 e1 = add2(f2(eci.x, eci.y), f2(ecj.x, ecj.y));   // (Pi11, Pi12)
-                    float e22 = eci.z + ecj.z;
-                    w = fma2(e1, bc(g.x), fma2(f2(e1.y, e22), bc(g.y), w));
+        LaneWords<LP, TURN> words(P, b, gi);
+        LaneTree<LP, TURN, 7> tree;
+#pragma unroll 1
+        for (int l = words.first(); l <= words.last(); l++) {
+            if (LP > 1) {
+                w = su = sd = f2(0.f, 0.f);
+                sr = 0.f;
+            }
+            words.template walk<ANN_PF_D>(l, [&](int o, int, unsigned in) {
+                float4 bj = slot_at(sb, o);
+                float2 d = pair_d(pi, slot_at(sp, o));
+                float r2 = len2(d);
+                KernelPowers kp = kernel_powers<true>(r2, P);
+                float Wv = kernel_w_of(kp, P), F = kernel_f_of(kp, P);
+                float2 du = sub2(ui, f2(bj.z, bj.w));   // u_i - u_j
+                float ud = fmaf(du.x, d.x, du.y * d.y);
+                float rinv2 = kp.rinv * kp.rinv;
+                if (CONS) {
+                    float2 cj = slot_at(sc, o);
+                    float2 g = mul2(bc(F), d);
+                    float visc = k8 * bj.y * ud * rinv2;
+                    w = fma2(bc(visc - (bi.x + bj.x)), g, w);
+                    float2 qs = add2(ci, cj);   // (Q11_i/rho_i^2 + Q11_j/rho_j^2, same for Q12)
+                    // Q.g = (qa gx + qb gy, qb gx - qa gy)
+                    float2 act = fma2(qs, bc(g.x), mul2(f2(qs.y, -qs.x), bc(g.y)));
+                    w = fma2(bc(-P.zeta), act, w);
+                    if (EL) {   // + sum_j m (Pi_i/rho_i^2 + Pi_j/rho_j^2) . grad_i W
+                        float4 ecj = slot_at(se, o);
+                        float2 e1 = add2(f2(eci.x, eci.y), f2(ecj.x, ecj.y));   // (Pi11, Pi12)
+                        float e22 = eci.z + ecj.z;
+                        w = fma2(e1, bc(g.x), fma2(f2(e1.y, e22), bc(g.y), w));
+                    }
+                } else {
+                    float coef = fmaf(kv, ud * rinv2, fmaf(nrho, bj.y, pci));
+                    w = fma2(bc(bj.x * F * coef), d, w);
                 }
-            } else {
-                float coef = fmaf(kv, ud * rinv2, fmaf(nrho, bj.y, pci));
-                w = fma2(bc(bj.x * F * coef), d, w);
-            }
-            su = fma2(du, bc(Wv), su);
-            // APD sums run over the neighbours only (their terms do not vanish at the support
-            // edge): `in` is the candidate's bit of the neighbour mask
-            if (in) {
-                sr += kp.r;
-                sd = fma2(d, bc(rinv2 * kp.rinv), sd);
-            }
-        });
-        if (LP > 1) {
+                su = fma2(du, bc(Wv), su);
+                // APD sums run over the neighbours only (their terms do not vanish at the support
+                // edge): `in` is the candidate's bit of the neighbour mask
+                if (in) {
+                    sr += kp.r;
+                    sd = fma2(d, bc(rinv2 * kp.rinv), sd);
+                }
+            });
+            tree.join(l, w, su, sd, sr);
+        }
+        if (LP > 1 && !TURN) {
             w = lane_sum<LP>(w);
             su = lane_sum<LP>(su);
             sd = lane_sum<LP>(sd);
             sr = lane_sum<LP>(sr);
-            if (!writes<LP>()) continue;
+            if (!writes<LP, TURN>()) continue;
         }
         const float4 bb = b.bk[gi], cc = b.cq[gi];
         float kri = bb.w, swi = cc.w;
@@ -1194,20 +1309,20 @@ __global__ void BOUNDS_D k_pass_d(DevParams P, Bufs b)
             ax = P.mass * w.x;
             ay = P.mass * w.y;
         } else {
-            ax = fmaf(B11, w.x, B12 * w.y) - P.zeta * irho * dvx + irho * elx;
-            ay = fmaf(B12, w.x, B22 * w.y) - P.zeta * irho * dvy + irho * ely;
+            ax = fmaf(irho, elx, fmaf(-__fmul_rn(P.zeta, irho), dvx, dot2(B11, w.x, B12, w.y)));
+            ay = fmaf(irho, ely, fmaf(-__fmul_rn(P.zeta, irho), dvy, dot2(B12, w.x, B22, w.y)));
         }
         float sux = su.x, suy = su.y, sdx = sd.x, sdy = sd.y;
-        float unx = bi.z + P.half_dt * ax, uny = bi.w + P.half_dt * ay;
+        float unx = fmaf(P.half_dt, ax, bi.z), uny = fmaf(P.half_dt, ay, bi.w);
         float apx = 0.f, apy = 0.f;
         if (P.apd && c > 0) {
-            float uv = sqrtf(sux * sux + suy * suy) / swi;
+            float uv = sqrtf(dot2(sux, sux, suy, suy)) / swi;
             float r0 = sr / (float)c;
             float sc_ = P.dt * uv * r0 * r0;
-            apx = sc_ * sdx;
-            apy = sc_ * sdy;
+            apx = __fmul_rn(sc_, sdx);
+            apy = __fmul_rn(sc_, sdy);
         }
-        float stepx = P.half_dt * unx + apx, stepy = P.half_dt * uny + apy;
+        float stepx = fmaf(P.half_dt, unx, apx), stepy = fmaf(P.half_dt, uny, apy);
         double xn = mxi + widen(stepx);
         double yn = myi + widen(stepy);
         if (!(in_box(xn, P.bitsL) && in_box(yn, P.bitsL))) {   // rare: re-insert (Eq. 30)
@@ -1561,46 +1676,46 @@ cudaError_t allow_smem(F *f, int bytes)
     return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
-template <int LP, int T>
+template <int LP, int T, bool TURN = false>
 cudaError_t prepare_passes()
 {
     cudaError_t e;
-    if ((e = allow_smem(k_pass_a_filter<LP, T>, SMEM_AF))) return e;
-    if ((e = allow_smem(k_pass_b<false, LP, T>, SMEM_B))) return e;
-    if ((e = allow_smem(k_pass_b<true, LP, T>, SMEM_B))) return e;
-    if ((e = allow_smem(k_pass_c<false, false, LP, T>, smem_c(false)))) return e;
-    if ((e = allow_smem(k_pass_c<true, false, LP, T>, smem_c(false)))) return e;
-    if ((e = allow_smem(k_pass_c<false, true, LP, T>, smem_c(true)))) return e;
-    if ((e = allow_smem(k_pass_c<true, true, LP, T>, smem_c(true)))) return e;
-    if ((e = allow_smem(k_pass_d<false, false, LP, T>, smem_d(false, false)))) return e;
-    if ((e = allow_smem(k_pass_d<true, false, LP, T>, smem_d(true, false)))) return e;
-    if ((e = allow_smem(k_pass_d<false, true, LP, T>, smem_d(false, true)))) return e;
-    return allow_smem(k_pass_d<true, true, LP, T>, smem_d(true, true));
+    if ((e = allow_smem(k_pass_a_filter<LP, T, TURN>, SMEM_AF))) return e;
+    if ((e = allow_smem(k_pass_b<false, LP, T, TURN>, SMEM_B))) return e;
+    if ((e = allow_smem(k_pass_b<true, LP, T, TURN>, SMEM_B))) return e;
+    if ((e = allow_smem(k_pass_c<false, false, LP, T, TURN>, smem_c(false)))) return e;
+    if ((e = allow_smem(k_pass_c<true, false, LP, T, TURN>, smem_c(false)))) return e;
+    if ((e = allow_smem(k_pass_c<false, true, LP, T, TURN>, smem_c(true)))) return e;
+    if ((e = allow_smem(k_pass_c<true, true, LP, T, TURN>, smem_c(true)))) return e;
+    if ((e = allow_smem(k_pass_d<false, false, LP, T, TURN>, smem_d(false, false)))) return e;
+    if ((e = allow_smem(k_pass_d<true, false, LP, T, TURN>, smem_d(true, false)))) return e;
+    if ((e = allow_smem(k_pass_d<false, true, LP, T, TURN>, smem_d(false, true)))) return e;
+    return allow_smem(k_pass_d<true, true, LP, T, TURN>, smem_d(true, true));
 }
 
 // Pass k (6 to 9) with LP lanes per particle.
-template <int LP, int T>
+template <int LP, int T, bool TURN = false>
 void launch_pass(int k, const DevParams &P, const Bufs &b, cudaStream_t s)
 {
-    const dim3 nt(P.tiles * LP, P.tiles);
+    const dim3 nt(P.tiles * (TURN ? 1 : LP), P.tiles);
     const bool el = P.elastic && !P.conservative;   // the paper momentum takes div Pi from pass C
     switch (k) {
-    case 6: k_pass_a_filter<LP, T><<<nt, T, SMEM_AF, s>>>(P, b); break;
+    case 6: k_pass_a_filter<LP, T, TURN><<<nt, T, SMEM_AF, s>>>(P, b); break;
     case 7:
-        if (P.qnew) k_pass_b<false, LP, T><<<nt, T, SMEM_B, s>>>(P, b);
-        else k_pass_b<true, LP, T><<<nt, T, SMEM_B, s>>>(P, b);
+        if (P.qnew) k_pass_b<false, LP, T, TURN><<<nt, T, SMEM_B, s>>>(P, b);
+        else k_pass_b<true, LP, T, TURN><<<nt, T, SMEM_B, s>>>(P, b);
         break;
     case 8:
-        if (P.qnew && el) k_pass_c<true, true, LP, T><<<nt, T, smem_c(true), s>>>(P, b);
-        else if (P.qnew) k_pass_c<true, false, LP, T><<<nt, T, smem_c(false), s>>>(P, b);
-        else if (el) k_pass_c<false, true, LP, T><<<nt, T, smem_c(true), s>>>(P, b);
-        else k_pass_c<false, false, LP, T><<<nt, T, smem_c(false), s>>>(P, b);
+        if (P.qnew && el) k_pass_c<true, true, LP, T, TURN><<<nt, T, smem_c(true), s>>>(P, b);
+        else if (P.qnew) k_pass_c<true, false, LP, T, TURN><<<nt, T, smem_c(false), s>>>(P, b);
+        else if (el) k_pass_c<false, true, LP, T, TURN><<<nt, T, smem_c(true), s>>>(P, b);
+        else k_pass_c<false, false, LP, T, TURN><<<nt, T, smem_c(false), s>>>(P, b);
         break;
     case 9:
-        if (P.conservative && P.elastic) k_pass_d<true, true, LP, T><<<nt, T, smem_d(true, true), s>>>(P, b);
-        else if (P.conservative) k_pass_d<true, false, LP, T><<<nt, T, smem_d(true, false), s>>>(P, b);
-        else if (P.elastic) k_pass_d<false, true, LP, T><<<nt, T, smem_d(false, true), s>>>(P, b);
-        else k_pass_d<false, false, LP, T><<<nt, T, smem_d(false, false), s>>>(P, b);
+        if (P.conservative && P.elastic) k_pass_d<true, true, LP, T, TURN><<<nt, T, smem_d(true, true), s>>>(P, b);
+        else if (P.conservative) k_pass_d<true, false, LP, T, TURN><<<nt, T, smem_d(true, false), s>>>(P, b);
+        else if (P.elastic) k_pass_d<false, true, LP, T, TURN><<<nt, T, smem_d(false, true), s>>>(P, b);
+        else k_pass_d<false, false, LP, T, TURN><<<nt, T, smem_d(false, false), s>>>(P, b);
         break;
     }
 }
@@ -1615,6 +1730,11 @@ cudaError_t prepare_kernels(const DevParams &P)
     else e = allow_smem(k_pass_a_resort<false, PT>, smem_a(PT));
     if (!e) e = allow_smem(k_pass_a_resort<true, PT>, smem_a(PT));
     if (e) return e;
+    if (P.in_turn) {
+        if (P.lanes == 8) return prepare_passes<8, PT_FEW, true>();
+        if (P.lanes == 4) return prepare_passes<4, PT_FEW, true>();
+        if (P.lanes == 2) return prepare_passes<2, PT_FEW, true>();
+    }
     if (P.lanes == 8) return prepare_passes<8, PT_FEW>();
     if (P.lanes == 4) return prepare_passes<4, PT_FEW>();
     if (P.lanes == 2) return prepare_passes<2, PT_FEW>();
@@ -1638,7 +1758,10 @@ cudaError_t launch_kernel(int k, const DevParams &P, const Bufs &b, cudaStream_t
         else k_pass_a_resort<false, PT><<<nt, PT, smem_a(PT), s>>>(P, b);
         break;
     case 6: case 7: case 8: case 9:
-        if (P.lanes == 8) launch_pass<8, PT_FEW>(k, P, b, s);
+        if (P.in_turn && P.lanes == 8) launch_pass<8, PT_FEW, true>(k, P, b, s);
+        else if (P.in_turn && P.lanes == 4) launch_pass<4, PT_FEW, true>(k, P, b, s);
+        else if (P.in_turn && P.lanes == 2) launch_pass<2, PT_FEW, true>(k, P, b, s);
+        else if (P.lanes == 8) launch_pass<8, PT_FEW>(k, P, b, s);
         else if (P.lanes == 4) launch_pass<4, PT_FEW>(k, P, b, s);
         else if (P.lanes == 2) launch_pass<2, PT_FEW>(k, P, b, s);
         else if (P.threads == PT_FEW) launch_pass<1, PT_FEW>(k, P, b, s);
