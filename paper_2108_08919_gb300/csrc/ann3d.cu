@@ -17,7 +17,7 @@
 //   pass 3      momentum (Eq. 23), artificial displacement (Eq. 29), corrector
 //
 // Tiles.  A pair kernel runs one block per non-empty cell (side >= 3h (1 + 0.05), ~70 particles on a
-// lattice).  The re-sort lists, for each cell, the particles of the 27 surrounding cells that come
+// lattice at h = 1.3 dx; wider where that would hold few, see cells3).  The re-sort lists, for each cell, the particles of the 27 surrounding cells that come
 // within the candidate radius of the box around the cell's own particles (~1,300 of ~1,900); a
 // pair kernel stages these "slots" in shared memory, with positions relative to the cell's centre,
 // and the candidate lists name slots: 16-bit byte offsets of 16-byte records, whose free bit 0 says
@@ -63,6 +63,7 @@ using ann::sub2;
 constexpr int MAXN3 = ANN3_MAX_NEIGHBORS;
 constexpr int MAXC3 = 576;          // candidates: neighbours within 3h (1 + SKIN3) at the last re-sort
 constexpr double CELL3 = 0.05;      // cells are at least 3h (1 + CELL3) wide
+constexpr double SPARSE3 = 50.0, GROW3 = 3.0;   // and wider, up to GROW3 times, where they would hold fewer than SPARSE3 particles: see cells3
 // Candidate lists stay valid while no particle moves SKIN3 3h / 2.  A skin of 0.02 keeps ~6 % more
 // candidates than neighbours (0.05: 16 %); a re-sort costs about one step and a half.
 constexpr double SKIN3 = 0.02;
@@ -89,7 +90,7 @@ struct P3 {
     int n, nc, ncell, nblk;      // nblk: blocks of a pair kernel, at least the non-empty cells
     double L, inv_cell, R2d, half_dt_d;
     long long bitsL;
-    float inv_h, ad, kw6, kw15, kf5, kf30, kf75, W0, dt, half_dt, cell_f, hL, R2lo, R2hi, R2c, far;   // hL: L / 2; far: beyond any tile and its support
+    float inv_h, ad, kw6, kw15, kf5, kf30, kf75, W0, dt, half_dt, cell_f, cell_lo, hL, R2lo, R2hi, R2c, far;   // hL: L / 2; far: beyond any tile and its support
     float skin_max2;
     float rho0, nu, Gamma, lambda, A, B, C, K, zeta, gamma_eos, beta, c0_min, c_shift;
     int apd;
@@ -302,6 +303,14 @@ __global__ void __launch_bounds__(256) k3_scatter(P3 P, Work3 w)
     if (i < P.n) w.perm[w.start[w.key[i]] + w.rank[i]] = i;
 }
 
+// Adds up, over the particles, how many particles share each one's cell (w.key and w.count of k3_keys).
+__global__ void __launch_bounds__(256) k3_crowd(int n, Work3 w, unsigned long long *sum)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned v = __reduce_add_sync(0xffffffffu, i < n ? (unsigned)w.count[w.key[i]] : 0u);
+    if ((threadIdx.x & 31) == 0) atomicAdd(sum, (unsigned long long)v);
+}
+
 // The slots of each cell in particle-ID order: a warp per cell ranks each particle among the cell's by
 // comparing IDs (all distinct), and moves its state to its place in T.
 __global__ void __launch_bounds__(256) k3_order(P3 P, const Set3 S, Set3 T, Work3 w)
@@ -359,11 +368,12 @@ __device__ __forceinline__ int halo_cell(const P3 &P, int cx, int cy, int cz, in
     return (qz * P.nc + qy) * P.nc + qx;
 }
 
-// Position relative to the tile's centre of a particle with offsets xi in halo cell o.
+// Position relative to the tile's centre of a particle with offsets xi in halo cell o (cell_lo: what FP32 drops of
+// the cell's side).
 __device__ __forceinline__ float4 tile_pos(const P3 &P, float4 xi, int o)
 {
-    return make_float4(fmaf((float)(o % 3 - 1), P.cell_f, xi.x), fmaf((float)(o / 3 % 3 - 1), P.cell_f, xi.y),
-                       fmaf((float)(o / 9 - 1), P.cell_f, xi.z), xi.w);
+    auto at = [&](int k, float x) { return fmaf((float)k, P.cell_f, fmaf((float)k, P.cell_lo, x)); };
+    return make_float4(at(o % 3 - 1, xi.x), at(o / 3 % 3 - 1, xi.y), at(o / 9 - 1, xi.z), xi.w);
 }
 
 __device__ __forceinline__ float dist2(float4 a, float4 b)
@@ -1214,6 +1224,8 @@ struct ann3_ctx {
     int64_t steps = 0;
     std::string last_err;
     double *tmp = nullptr;         // device staging for ann3_get_field (9n doubles)
+    int nc_fine = 0;               // cells a side at their least width
+    double *centre = nullptr;      // Work3::centre, nc_fine values
 };
 
 namespace {
@@ -1311,6 +1323,81 @@ cudaError_t capture3(ann3_ctx *c)
     return ec ? ec : e;
 }
 
+// Cells a side for n particles that share a cell of the least width with m particles on average, themselves included.
+// A pair kernel's block pays for its launch and for staging a cell's halo whatever the cell holds, so with cells
+// of few particles (h below ~1.15 dx) a step got dearer the fewer neighbours there were.  There the cells are
+// widened until they hold 50 particles, or up to 216 where that leaves 700 tiles (a tile then stages at most
+// ~1,900 of the 2,199 slots).  us a step with cells of the least width / these / one thread a particle and no tiles:
+// 80^3 at h = 0.5 dx 6,759 / 536 / 433, 0.6 4,152 / 474 / 501, 0.8 2,262 / 672 / 818, 1.0 1,629 / 885 / 1,214, 1.1 1,580 /
+// 1,088 / 1,589; 48^3 at 0.5 993 / 123 / 131, 0.8 384 / 176 / 227, 1.0 299 / 232 / 328; 24^3 at 0.5 148 / 44 / 84, 0.9 62 / 56 /
+// 146.  From m = 50 on (1.15 dx) nothing changes.  m is an average over the particles, not over the box: a
+// dense patch in an empty box keeps the cells that fit it.  At most GROW3 times the least width: positions are FP32
+// offsets within a tile, up to 4.7 h with the least cells and 7.8 h with these, which leaves the fields' errors against
+// FP64 at 0.7 to 1.4 times (~3e-7 of the field) and r^2 of a pair good to 2.1e-6, inside the band that FP64 decides.
+int cells3(int nc_fine, int64_t n, double m)
+{
+    if (m >= SPARSE3) return nc_fine;
+    const double want = std::min(std::max((double)n / 700.0, SPARSE3), 216.0);
+    const int nc = std::max(3, (int)std::lround(nc_fine / std::min(GROW3, std::cbrt(want / m))));
+    return nc == 7 ? 6 : nc;   // 343 tiles: a second wave of 39 on the 304 blocks that run at once
+}
+
+// nc cells a side: the parameters that depend on it, and the cells' centres.
+cudaError_t set_cells3(ann3_ctx *c, int nc)
+{
+    P3 &P = c->P;
+    const double cell = c->prm.L / nc;
+    P.nc = nc;
+    P.ncell = nc * nc * nc;
+    P.nblk = std::min(P.ncell, P.n);
+    P.inv_cell = nc / c->prm.L;
+    P.cell_f = (float)cell;
+    P.cell_lo = (float)(cell - (double)P.cell_f);
+    P.far = (float)(64.0 * cell);
+    std::vector<double> centre((size_t)nc);
+    for (int k = 0; k < nc; k++) centre[(size_t)k] = (k + 0.5) * cell;
+    const cudaError_t e =
+        cudaMemcpyAsync(c->centre, centre.data(), sizeof(double) * (size_t)nc, cudaMemcpyHostToDevice, c->s);
+    return e ? e : cudaStreamSynchronize(c->s);
+}
+
+// Gives the box nc cells a side and captures the step anew if that is not what it has.
+cudaError_t regrid3(ann3_ctx *c, int nc)
+{
+    if (nc == c->P.nc) return cudaSuccess;
+    const int was = c->P.nc;
+    cudaGraphExec_t old = c->exec;
+    cudaError_t e = set_cells3(c, nc);
+    if (!e) e = capture3(c);
+    if (e) {   // as it was
+        c->exec = old;
+        set_cells3(c, was);
+        return e;
+    }
+    return cudaGraphExecDestroy(old);
+}
+
+// Sizes the cells for the state loaded in S: counts it into cells of the least width, unless these hold SPARSE3 over
+// the whole box and so, or more, over the particles.
+cudaError_t fit_cells3(ann3_ctx *c)
+{
+    P3 fine = c->P;
+    fine.nc = c->nc_fine;
+    fine.inv_cell = c->nc_fine / c->prm.L;
+    const size_t n = (size_t)fine.n, ncell = (size_t)fine.nc * fine.nc * fine.nc;
+    if ((double)n / (double)ncell >= SPARSE3) return regrid3(c, fine.nc);
+    unsigned long long crowd = 0, *sum = reinterpret_cast<unsigned long long *>(c->tmp);
+    cudaError_t e = cudaMemsetAsync(sum, 0, sizeof crowd, c->s);
+    if (e) return e;
+    k3_keys<<<nb3(n), 256, 0, c->s>>>(fine, c->S, c->w);
+    k3_crowd<<<nb3(n), 256, 0, c->s>>>(fine.n, c->w, sum);
+    e = cudaGetLastError();
+    if (!e) e = cudaMemcpyAsync(&crowd, sum, sizeof crowd, cudaMemcpyDeviceToHost, c->s);
+    if (!e) e = cudaMemsetAsync(c->w.count, 0, sizeof(int) * ncell, c->s);   // as the re-sort leaves them
+    if (!e) e = cudaStreamSynchronize(c->s);
+    return e ? e : regrid3(c, cells3(c->nc_fine, fine.n, (double)crowd / (double)n));
+}
+
 int fail3(ann3_ctx *c, int code, const std::string &m)
 {
     if (c) c->last_err = m;
@@ -1376,17 +1463,12 @@ int ann3_create(const ann3_params *p, ann3_ctx **out)
     if (!c) return ANN_ERR_OOM;
     c->prm = *p;
     P3 &P = c->P;
+    c->nc_fine = nc;
+    const size_t ncell = (size_t)nc * nc * nc;
     P.n = (int)p->n;
-    P.nc = nc;
-    P.ncell = nc * nc * nc;
-    P.nblk = std::min(P.ncell, P.n);
     P.L = p->L;
     std::memcpy(&P.bitsL, &p->L, sizeof P.bitsL);
-    P.inv_cell = nc / p->L;
-    const double cell = p->L / nc;
-    P.cell_f = (float)cell;
     P.hL = (float)(0.5 * p->L);
-    P.far = (float)(64.0 * cell);
     P.R2d = 9.0 * p->h * p->h;
     P.R2lo = (float)(P.R2d * (1.0 - 4e-6));   // FP32 r^2 of a pair is good to ~1e-6 relative
     P.R2hi = (float)(P.R2d * (1.0 + 4e-6));
@@ -1427,9 +1509,9 @@ int ann3_create(const ann3_params *p, ann3_ctx **out)
     if (!e) e = alloc3(c, w.key, n);
     if (!e) e = alloc3(c, w.rank, n);
     if (!e) e = alloc3(c, w.perm, n);
-    if (!e) e = alloc3(c, w.count, (size_t)P.ncell);
-    if (!e) e = alloc3(c, w.start, (size_t)P.ncell + 1);
-    if (!e) e = alloc3(c, w.tile, (size_t)P.nblk);
+    if (!e) e = alloc3(c, w.count, ncell);
+    if (!e) e = alloc3(c, w.start, ncell + 1);
+    if (!e) e = alloc3(c, w.tile, std::min(ncell, n));
     if (!e) e = alloc3(c, w.ntile, 1);
     if (!e) e = alloc3(c, w.slots_used, 1);
     if (!e) e = alloc3(c, w.slot, 27 * n);
@@ -1460,12 +1542,9 @@ int ann3_create(const ann3_params *p, ann3_ctx **out)
     if (!e) e = alloc3(c, w.umax, 1);
     if (!e) e = alloc3(c, w.err, 1);
     if (!e) e = alloc3(c, c->tmp, 9 * n);
-    double *centre = nullptr;
-    if (!e) e = alloc3(c, centre, (size_t)nc);
-    std::vector<double> hc((size_t)nc);
-    for (int k = 0; k < nc; k++) hc[(size_t)k] = (k + 0.5) * cell;
-    if (!e) e = cudaMemcpyAsync(centre, hc.data(), sizeof(double) * (size_t)nc, cudaMemcpyHostToDevice, c->s);
-    w.centre = centre;
+    if (!e) e = alloc3(c, c->centre, (size_t)nc);
+    w.centre = c->centre;
+    if (!e) e = set_cells3(c, nc);
     if (!e) e = cudaFuncSetAttribute(k3_pass1, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM3_1);
     if (!e) e = cudaFuncSetAttribute(k3_pass2, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM3_2);
     if (!e) e = cudaFuncSetAttribute(k3_pass3, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM3_3);
@@ -1532,6 +1611,7 @@ int ann3_set_particles(ann3_ctx *c, int64_t n, const double *x, const double *y,
     if (!e) e = cudaMemcpyAsync(c->w.flag, &one, 4, cudaMemcpyHostToDevice, c->s);
     if (!e) e = cudaMemsetAsync(c->w.rebuilds, 0, 4, c->s);
     if (!e) e = cudaStreamSynchronize(c->s);
+    if (!e) e = fit_cells3(c);
     if (e) return cuda3(c, e, "ann3_set_particles");
     c->have = true;
     c->steps = 0;
