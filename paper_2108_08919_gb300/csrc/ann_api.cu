@@ -1763,7 +1763,10 @@ cudaError_t build_ensemble_graph(ann_ensemble *E, int groups)
         P.push_back(c->P);
         P.back().threads = threads_for((int)std::min<int64_t>(side_by_side(tiles, own_tiles), 1 << 30));
         P.back().in_turn = lanes_in_turn(own, side_by_side(threads, own));
-        if (!e) e = prepare_kernels(P.back());
+        bool ready = false;   // by an earlier member launched alike
+        for (size_t k = 0; k + 1 < P.size(); k++)
+            ready |= P[k].lanes == P.back().lanes && P[k].threads == P.back().threads && P[k].in_turn == P.back().in_turn;
+        if (!e && !ready) e = prepare_kernels(P.back());
     }
     if (e) return e;
     cudaGraph_t g = nullptr;
