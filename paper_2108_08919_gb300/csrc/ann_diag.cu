@@ -316,31 +316,34 @@ __device__ __forceinline__ int crossing(double a1, double a2, double b1, double 
 // takes each edge once, through shared memory.  The kernel is bound by FP64 issue (2 a cycle and
 // SM); the counts are summed per block.  M = 1024: 32 us, where taking four edges a
 // plaquette with an atomic per defect took 74.
-constexpr int DEF_ROWS = 8;
+// Grids below 256 nodes a side, whose blocks would be too few or too narrow to hide a column's eight
+// rows, take a row a block (a call at M = 8: 20.5 us with four edges a plaquette, 28.8 with eight rows a block).
+constexpr int DEF_ROWS = 8, DEF_FEW = 256;
 
+template <int ROWS>
 __global__ void __launch_bounds__(256) k_defects(int M, const double *grid, signed char *map, unsigned long long *counts)
 {
-    __shared__ signed char up[DEF_ROWS][257];   // edge (ix, iy) -> (ix, iy + 1)
+    __shared__ signed char up[ROWS][257];   // edge (ix, iy) -> (ix, iy + 1)
     __shared__ int sum[3];
     const size_t MM = (size_t)M * M;
     const double *q1 = grid + 2 * MM, *q2 = grid + 3 * MM;
     const int W = blockDim.x, x0 = blockIdx.x * W, ix = x0 + threadIdx.x, xp = (ix + 1) & (M - 1);
-    const int y0 = blockIdx.y * DEF_ROWS, xe = (x0 + W) & (M - 1);   // M is a power of two, at least 8
+    const int y0 = blockIdx.y * ROWS, xe = (x0 + W) & (M - 1);   // M is a power of two, at least 8
     if (threadIdx.x < 3) sum[threadIdx.x] = 0;
-    int right[DEF_ROWS + 1];   // edge (ix, iy) -> (ix + 1, iy)
+    int right[ROWS + 1];   // edge (ix, iy) -> (ix + 1, iy)
     double a1 = q1[(size_t)y0 * M + ix], a2 = q2[(size_t)y0 * M + ix];
 #pragma unroll
-    for (int r = 0; r <= DEF_ROWS; r++) {
+    for (int r = 0; r <= ROWS; r++) {
         const size_t row = (size_t)((y0 + r) & (M - 1)) * M;
         right[r] = crossing(a1, a2, q1[row + xp], q2[row + xp]);
-        if (r == DEF_ROWS) break;
+        if (r == ROWS) break;
         const size_t nxt = (size_t)((y0 + r + 1) & (M - 1)) * M + ix;
         const double b1 = q1[nxt], b2 = q2[nxt];
         up[r][threadIdx.x] = (signed char)crossing(a1, a2, b1, b2);
         a1 = b1;
         a2 = b2;
     }
-    if (threadIdx.x < DEF_ROWS) {   // the column past the block's last
+    if (threadIdx.x < ROWS) {   // the column past the block's last
         const size_t g = (size_t)(y0 + threadIdx.x) * M + xe;
         const size_t h = (size_t)((y0 + threadIdx.x + 1) & (M - 1)) * M + xe;
         up[threadIdx.x][W] = (signed char)crossing(q1[g], q2[g], q1[h], q2[h]);
@@ -348,7 +351,7 @@ __global__ void __launch_bounds__(256) k_defects(int M, const double *grid, sign
     __syncthreads();
     int plus = 0, minus = 0, more = 0;
 #pragma unroll
-    for (int r = 0; r < DEF_ROWS; r++) {
+    for (int r = 0; r < ROWS; r++) {
         const int m = right[r] + up[r][threadIdx.x + 1] - right[r + 1] - up[r][threadIdx.x];
         map[(size_t)(y0 + r) * M + ix] = (signed char)m;
         plus += m == 1;
@@ -448,7 +451,8 @@ cudaError_t enqueue_defects(int M, const double *grid, signed char *map, unsigne
     cudaError_t e = cudaMemsetAsync(counts, 0, 3 * sizeof(unsigned long long), s);
     if (e) return e;
     const int w = M < 256 ? M : 256;
-    k_defects<<<dim3(M / w, M / DEF_ROWS), w, 0, s>>>(M, grid, map, counts);
+    if (M < DEF_FEW) k_defects<1><<<dim3(M / w, M), w, 0, s>>>(M, grid, map, counts);
+    else k_defects<DEF_ROWS><<<dim3(M / w, M / DEF_ROWS), w, 0, s>>>(M, grid, map, counts);
     return cudaGetLastError();
 }
 
