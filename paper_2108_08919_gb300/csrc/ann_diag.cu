@@ -249,32 +249,44 @@ __global__ void __launch_bounds__(256) k_shell_sum(int M, const double2 *Z, cons
 // Vorticity on the centre row by periodic central differences, and its correlation (Eq. 32).
 // ------------------------------------------------------------------------------------------------
 
-__global__ void __launch_bounds__(256) k_vorticity_row(int M, double L, const double *grid, double *om)
+__device__ __forceinline__ double vorticity(int M, double L, const double *grid, int i)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= M) return;
     const size_t MM = (size_t)M * M;
     const double *ux = grid, *uy = grid + MM;
     const int j0 = M / 2, jm = j0 - 1, jp = (j0 + 1) % M, ip = (i + 1) % M, im = (i + M - 1) % M;
     const double D2 = 2.0 * (L / M);
     const double dvx = (uy[(size_t)j0 * M + ip] - uy[(size_t)j0 * M + im]) / D2;
     const double duy = (ux[(size_t)jp * M + i] - ux[(size_t)jm * M + i]) / D2;
-    om[i] = dvx - duy;
+    return dvx - duy;
+}
+
+__global__ void __launch_bounds__(256) k_vorticity_row(int M, double L, const double *grid, double *om)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < M) om[i] = vorticity(M, L, grid, i);
 }
 
 // One warp per lag k: lane l sums the origins l, l + 32, ... and a fixed tree joins the lanes.  The
 // 2 M (M/2 + 1) multiply-adds are FP64 (2 a cycle and SM), so they are spread over the whole GPU: at
 // M = 1024 this takes 9 us and the row kernel 4 us, where one block with a thread per lag took 283 us.
-constexpr int CORR_WARPS = 4;
+// ONE: where there is little to sum (one origin, or a row of at most 64 nodes) one block takes the row too: a
+// second launch would cost more than it saves (a call 30.4 us with one kernel, 31.7 with two).
+constexpr int CORR_WARPS = 4, CORR_ONE = 64;
 
-__global__ void __launch_bounds__(32 * CORR_WARPS) k_correlation(int M, const double *row, int all_origins, double *C)
+template <bool ONE>
+__global__ void __launch_bounds__(ONE ? 1024 : 32 * CORR_WARPS)
+    k_correlation(int M, double L, const double *grid, const double *row, int all_origins, double *C)
 {
     extern __shared__ double om[];
-    for (int i = threadIdx.x; i < M; i += blockDim.x) om[i] = row[i];
+    for (int i = threadIdx.x; i < M; i += blockDim.x) om[i] = ONE ? vorticity(M, L, grid, i) : row[i];
     __syncthreads();
-    const int k = blockIdx.x * CORR_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (k > M / 2) return;
-    if (all_origins) {
+    if (ONE && !all_origins) {
+        const int i0 = M / 2;
+        for (int k = threadIdx.x; k <= M / 2; k += blockDim.x) C[k] = om[(i0 + k) & (M - 1)] * om[i0] / (om[i0] * om[i0]);
+        return;
+    }
+    const int warps = blockDim.x >> 5, lane = threadIdx.x & 31;
+    for (int k = blockIdx.x * warps + (threadIdx.x >> 5); k <= M / 2; k += ONE ? warps : M) {
         double num = 0.0, den = 0.0;
         for (int i = lane; i < M; i += 32) {
             num += om[(i + k) & (M - 1)] * om[i];   // M is a power of two
@@ -285,9 +297,6 @@ __global__ void __launch_bounds__(32 * CORR_WARPS) k_correlation(int M, const do
             den += __shfl_xor_sync(0xffffffffu, den, o);
         }
         if (lane == 0) C[k] = num / den;
-    } else if (lane == 0) {
-        const int i0 = M / 2;
-        C[k] = om[(i0 + k) & (M - 1)] * om[i0] / (om[i0] * om[i0]);
     }
 }
 
@@ -441,8 +450,12 @@ cudaError_t enqueue_correlation(int M, double L, const double *grid, int all_ori
                                 cudaStream_t s)
 {
     size_t smem = sizeof(double) * (size_t)M;
-    k_vorticity_row<<<blocks(M, 256), 256, 0, s>>>(M, L, grid, om);
-    k_correlation<<<blocks(M / 2 + 1, CORR_WARPS), 32 * CORR_WARPS, smem, s>>>(M, om, all_origins, C);
+    if (!all_origins || M <= CORR_ONE) {
+        k_correlation<true><<<1, 1024, smem, s>>>(M, L, grid, om, all_origins, C);
+    } else {
+        k_vorticity_row<<<blocks(M, 256), 256, 0, s>>>(M, L, grid, om);
+        k_correlation<false><<<blocks(M / 2 + 1, CORR_WARPS), 32 * CORR_WARPS, smem, s>>>(M, L, grid, om, all_origins, C);
+    }
     return cudaGetLastError();
 }
 
