@@ -153,7 +153,7 @@ __device__ __forceinline__ void butterfly(double2 a, double2 b, double2 w, doubl
 __host__ __device__ constexpr int fft_pad(int i) { return i + (i >> 2); }
 
 template <bool PACK>
-__global__ void __launch_bounds__(512) k_fft_rows(int M, int logM, const double2 *in, const double *gx, const double *gy,
+__global__ void __launch_bounds__(512) k_fft_rows(int M, const double2 *in, const double *gx, const double *gy,
                                                   double2 *out, const double2 *tw)
 {
     extern __shared__ double2 sm[];
@@ -430,18 +430,16 @@ cudaError_t enqueue_twiddles(int M, double2 *tw, cudaStream_t s)
 cudaError_t enqueue_spectrum(int M, const double *grid, double2 *z, double2 *zt, const double2 *tw,
                              const int *shell_off, const int *shell_modes, int nshell, double *E, cudaStream_t s)
 {
-    int logM = 0;
-    while ((1 << logM) < M) logM++;
     const int th = M / 4;   // 2 (M = 8) to 512
     size_t smem = sizeof(double2) * 2 * (size_t)fft_pad(M);
     cudaError_t e = cudaFuncSetAttribute(k_fft_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (!e) e = cudaFuncSetAttribute(k_fft_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e) return e;
     size_t MM = (size_t)M * M;
-    k_fft_rows<true><<<M, th, smem, s>>>(M, logM, nullptr, grid, grid + MM, z, tw);
+    k_fft_rows<true><<<M, th, smem, s>>>(M, nullptr, grid, grid + MM, z, tw);
     dim3 tb(32, 8), tg((M + 31) / 32, (M + 31) / 32);
     k_transpose<<<tg, tb, 0, s>>>(M, z, zt);
-    k_fft_rows<false><<<M, th, smem, s>>>(M, logM, zt, nullptr, nullptr, z, tw);
+    k_fft_rows<false><<<M, th, smem, s>>>(M, zt, nullptr, nullptr, z, tw);
     k_shell_sum<<<nshell, 256, 0, s>>>(M, z, shell_off, shell_modes, E);
     return cudaGetLastError();
 }

@@ -250,12 +250,11 @@ int ctx_commit_in_place(ann_ctx *c, int64_t add_steps);              // S was re
 
 // BF16 tensor-core GEMMs of the surrogate (ann_mlp.cu).  K, N multiples of 16 in [16, 256].
 bool gemm_shape_ok(int K, int N);
-// ldc: row stride of C in elements (0: N)
 cudaError_t enqueue_gemm_nt(const void *A1, int K1, const void *A2, int K2, const void *B, int N, int rows,
                             const float *bias, int relu, void *C, int c_bf16, int accumulate, unsigned *err,
-                            int max_ctas, cudaStream_t s, int ldc = 0);
+                            int max_ctas, cudaStream_t s);
 cudaError_t enqueue_gemm_tn(const void *A, int K, const void *B, int N, int rows, float *C, unsigned *err,
-                            int max_ctas, cudaStream_t s, int ldc = 0);
+                            int max_ctas, cudaStream_t s);
 // One surrogate layer: h = relu([A1 | A2] W^T + bw) (128 wide; to H unless null), z = h P^T + bp
 // (Np wide, bp may be null; BF16 or FP32).  W 128 x (K1 + K2), P Np x 128, BF16, 16-byte aligned.
 cudaError_t enqueue_layer(const void *A1, int K1, const void *A2, int K2, const void *W, const float *bw,

@@ -208,8 +208,8 @@ struct NtArgs {
     const __nv_bfloat16 *A1, *A2;   // rows x K1, rows x K2 (row-major), A2 may be null (K2 = 0)
     const __nv_bfloat16 *B;         // N x K (row-major: K-major)
     const float *bias;              // N or null
-    void *C;                        // rows x N (row stride ldc): BF16 or FP32
-    int rows, K1, K2, N, relu, c_bf16, accumulate, ldc;
+    void *C;                        // rows x N: BF16 or FP32
+    int rows, K1, K2, N, relu, c_bf16, accumulate;
     unsigned *err;
 };
 
@@ -278,11 +278,11 @@ __global__ void __launch_bounds__(128) k_gemm_nt(NtArgs a)
                     __nv_bfloat162 *h = reinterpret_cast<__nv_bfloat162 *>(w);
 #pragma unroll
                     for (int k = 0; k < 8; k++) h[k] = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
-                    uint4 *C = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(a.C) + (size_t)gr * a.ldc + c0);
+                    uint4 *C = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(a.C) + (size_t)gr * a.N + c0);
                     C[0] = w[0];
                     C[1] = w[1];
                 } else {          // 64 bytes: four 16-byte stores
-                    float4 *C = reinterpret_cast<float4 *>(static_cast<float *>(a.C) + (size_t)gr * a.ldc + c0);
+                    float4 *C = reinterpret_cast<float4 *>(static_cast<float *>(a.C) + (size_t)gr * a.N + c0);
 #pragma unroll
                     for (int k = 0; k < 4; k++) {
                         float4 o = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
@@ -700,8 +700,8 @@ __device__ __forceinline__ void stage_rows_T(const __nv_bfloat16 *X, int K, int 
 struct TnArgs {
     const __nv_bfloat16 *A;   // rows x K
     const __nv_bfloat16 *B;   // rows x N
-    float *C;                 // K x N (FP32, accumulated, row stride ldc)
-    int rows, K, N, ldc;
+    float *C;                 // K x N (FP32, accumulated)
+    int rows, K, N;
     unsigned *err;
 };
 
@@ -759,7 +759,7 @@ __global__ void __launch_bounds__(128) k_gemm_tn(TnArgs a)
             tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
             if (f < a.K)
 #pragma unroll
-                for (int k = 0; k < 16; k++) atomicAdd(&a.C[(size_t)f * a.ldc + c0 + k], v[k]);
+                for (int k = 0; k < 16; k++) atomicAdd(&a.C[(size_t)f * a.N + c0 + k], v[k]);
         }
     }
     fence_before();
@@ -942,11 +942,10 @@ bool gemm_shape_ok(int K, int N) { return K >= 16 && K <= 256 && K % 16 == 0 && 
 
 cudaError_t enqueue_gemm_nt(const void *A1, int K1, const void *A2, int K2, const void *B, int N, int rows,
                             const float *bias, int relu, void *C, int c_bf16, int accumulate, unsigned *err,
-                            int max_ctas, cudaStream_t s, int ldc)
+                            int max_ctas, cudaStream_t s)
 {
     NtArgs a{static_cast<const __nv_bfloat16 *>(A1), static_cast<const __nv_bfloat16 *>(A2),
-             static_cast<const __nv_bfloat16 *>(B), bias, C, rows, K1, K2, N, relu, c_bf16, accumulate,
-             ldc > 0 ? ldc : N, err};
+             static_cast<const __nv_bfloat16 *>(B), bias, C, rows, K1, K2, N, relu, c_bf16, accumulate, err};
     int K = K1 + K2;
     size_t smem = (size_t)(N + MT) * K * 2;
     cudaError_t e = cudaFuncSetAttribute(k_gemm_nt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1100,10 +1099,9 @@ cudaError_t enqueue_wgrad_sum(const WgradOut &o, cudaStream_t s)
 }
 
 cudaError_t enqueue_gemm_tn(const void *A, int K, const void *B, int N, int rows, float *C, unsigned *err,
-                            int max_ctas, cudaStream_t s, int ldc)
+                            int max_ctas, cudaStream_t s)
 {
-    TnArgs a{static_cast<const __nv_bfloat16 *>(A), static_cast<const __nv_bfloat16 *>(B), C, rows, K, N,
-             ldc > 0 ? ldc : N, err};
+    TnArgs a{static_cast<const __nv_bfloat16 *>(A), static_cast<const __nv_bfloat16 *>(B), C, rows, K, N, err};
     size_t smem = (size_t)(MT + N) * MT * 2;
     cudaError_t e = cudaFuncSetAttribute(k_gemm_tn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e) return e;
