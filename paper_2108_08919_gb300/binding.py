@@ -707,7 +707,7 @@ def _tend(tend):
 def ann_surrogate_load(sg, ctx, tend=None) -> None:
     """tend: None (the context's last recorded step) or (n, 8) tendencies in ID order."""
     if tend is not None and np.ndim(tend) == 2 and np.shape(tend)[1] == 8:
-        ann_surrogate_load_rows(sg, ctx, tend)
+        _load_rows(sg, ctx, tend, "ann_surrogate_load")
         return
     ptr, keep = _tend(tend)
     _scheck(lib().ann_surrogate_load(sg, ctx, ptr), sg, "ann_surrogate_load")
@@ -715,8 +715,12 @@ def ann_surrogate_load(sg, ctx, tend=None) -> None:
 
 def ann_surrogate_load_rows(sg, ctx, tend) -> None:
     """ann_surrogate_load with (n, 8) tendencies in ID order, which the device sorts into components."""
+    _load_rows(sg, ctx, tend, "ann_surrogate_load_rows")
+
+
+def _load_rows(sg, ctx, tend, what):
     rows = np.ascontiguousarray(tend, dtype=np.float32)
-    _scheck(lib().ann_surrogate_load_rows(sg, ctx, _fp(rows)), sg, "ann_surrogate_load")
+    _scheck(lib().ann_surrogate_load_rows(sg, ctx, _fp(rows)), sg, what)
 
 
 def ann_surrogate_forward(sg, n: int):
