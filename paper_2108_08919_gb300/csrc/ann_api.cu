@@ -183,18 +183,19 @@ int lanes_for(int tiles)
     return lanes;
 }
 
-// Whether an ensemble gives a member's particles one thread each, which takes the lanes in turn.  own, side_by_side:
-// particles x lanes of the member, and of all members that run at once.  Lanes on threads of their own shorten
-// a member's chain but cost the GPU more (LP halos staged, LP epilogues, shuffles), so they pay until the threads
-// fill the SMs about eight blocks deep (two rounds of four), and beyond that only where the member's passes
-// are so short that the launches bound them (one block an SM).  Measured, us a step with threads of their own /
+// Whether an ensemble gives a member's particles one thread each, which takes the lanes in turn.  mean, side_by_side:
+// particles x lanes of a member on average, and of this member and those that run with it.  Lanes on threads of
+// their own shorten a member's chain but cost the GPU more (LP halos staged, LP epilogues, shuffles), so they pay until
+// the threads fill the SMs about eight blocks deep (two rounds of four), and beyond that only where the members'
+// passes are so small that their launches are the bound (one block an SM).  Measured, us a step with threads of their own /
 // in turn / one lane, whose sums would not be a solo run's (members side by side): 64^2 x 4 65 / 76 / 71,
 // x 16 148 / 152 / 139; 96^2 x 4 77 / 78 / -, x 6 101 / 88 / -, x 16 230 / 166 / 149; 70^2 x 16 173 / 187 / -; 76^2
-// x 16 176 / 161 / -; 128^2 x 4 77 / 80 / 76, x 16 245 / 192 / 176; 192^2 x 16 353 / 293 / 275.
-bool lanes_in_turn(int64_t own, int64_t side_by_side)
+// x 16 176 / 161 / -; 128^2 x 4 77 / 80 / 76, x 16 245 / 192 / 176; 192^2 x 16 353 / 293 / 275; 32 members of 40^2 to
+// 130^2, mean 43,089, in 16 branches 355 / 383 / 330; of 48^2 to 256^2, mean 49,471, 550 / 497 / 488.
+bool lanes_in_turn(int64_t mean, int64_t side_by_side)
 {
     const int64_t block_an_sm = 152 * PT_FEW;
-    return own > block_an_sm && side_by_side > 8 * block_an_sm;
+    return mean > block_an_sm && side_by_side > 8 * block_an_sm;
 }
 
 // Threads per block of the pair passes.  A cell is at least 3h (1 + skin) wide, 3.98 spacings at h = 1.3 dx,
@@ -203,7 +204,10 @@ bool lanes_in_turn(int64_t own, int64_t side_by_side)
 // slowest tile is the pass: one round of 288 threads, at 4 blocks an SM instead of 5, took (us a step)
 // 104 -> 89 at 441 tiles (333^2, conservative), 71 -> 67 at 256 (256^2), 142 -> 139 at 1,024, 189 -> 184
 // at 1,444; with 4,225 (1024^2) the waves hide the second round, and the fifth block is worth more:
-// 447 -> 456, and 6,129 -> 6,290 at 4096^2.  320 threads: 90 at 441 tiles, 465 at 4,225.
+// 447 -> 456, and 6,129 -> 6,290 at 4096^2.  320 threads: 90 at 441 tiles, 465 at 4,225.  Away from h = 1.3 dx, where
+// a tile holds 97 (0.8 dx) to 300 (1.4), 256 / 288 threads take: 256^2 at 0.8 / 1.0 / 1.2 / 1.35 dx 54 / 69 / 83 /
+// 104 against 62 / 66 / 81 / 94, 333^2 72 / 82 / 97 / 123 against 70 / 86 / 95 / 113, 512^2 118 / 131 / 158 / 210 against
+// 120 / 132 / 159 / 184: the wider blocks mostly pay there too, so the line is drawn by the tiles alone.
 int threads_for(int tiles) { return tiles <= 1520 ? PT_FEW : PT; }   // ten tiles an SM
 
 DevParams make_dev(const ann_params &p)
@@ -1750,19 +1754,20 @@ cudaError_t build_ensemble_graph(ann_ensemble *E, int groups)
     // The wider blocks pay where all tiles run at once, here those of `groups` members side by side: 64
     // members of 128^2 to 512^2 take 2.98 ms a step in 16 branches and in 64 with 256 threads, 3.07 and 3.10
     // with 288.  A particle's sums are the same either way, so members stay bit-identical to solo runs.
-    int64_t tiles = 0, threads = 0;
+    const int64_t members = (int64_t)E->m.size();
+    int64_t tiles = 0, mean = 0;
     for (const ann_ctx *c : E->m) {
         tiles += (int64_t)c->P.tiles * c->P.tiles;
-        threads += (int64_t)c->P.n * c->P.lanes;
+        mean += (int64_t)c->P.n * c->P.lanes;
     }
-    auto side_by_side = [&](int64_t all, int64_t own) { return std::max(all * groups / (int64_t)E->m.size(), own); };
+    mean /= members;
     std::vector<DevParams> P;
     cudaError_t e = cudaSuccess;
     for (const ann_ctx *c : E->m) {
-        const int64_t own_tiles = (int64_t)c->P.tiles * c->P.tiles, own = (int64_t)c->P.n * c->P.lanes;
+        const int64_t side_by_side = std::max(tiles * groups / members, (int64_t)c->P.tiles * c->P.tiles);
         P.push_back(c->P);
-        P.back().threads = threads_for((int)std::min<int64_t>(side_by_side(tiles, own_tiles), 1 << 30));
-        P.back().in_turn = lanes_in_turn(own, side_by_side(threads, own));
+        P.back().threads = threads_for((int)std::min<int64_t>(side_by_side, 1 << 30));
+        P.back().in_turn = lanes_in_turn(mean, (int64_t)c->P.n * c->P.lanes + mean * (groups - 1));
         bool ready = false;   // by an earlier member launched alike
         for (size_t k = 0; k + 1 < P.size(); k++)
             ready |= P[k].lanes == P.back().lanes && P[k].threads == P.back().threads && P[k].in_turn == P.back().in_turn;
