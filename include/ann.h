@@ -610,8 +610,9 @@ int ann_velocity_moments_noalloc(const float *ux, const float *uy, const float *
  * side L; cells of side >= 3h (1 + 0.05), at least 3 per side (L >= 9.45 h: 13 particles a side at
  * h = 1.3 dx).  Candidate lists (every j within 3h (1 + 0.02), rebuilt with a re-sort when a
  * particle has moved 0.02 x 3h / 2) hold at most 576, neighbour lists ANN3_MAX_NEIGHBORS (~250 at
- * h = 1.3 dx).  FP64 positions; pair differences are taken
- * in FP64 and everything else runs in FP32.  The step order is that of the 2D step (modified
+ * h = 1.3 dx).  The cells are wider, up to three times, where a loaded state leaves them few particles.  FP64
+ * positions; pair differences and everything else run in FP32, on offsets from the centre of a cell, and a pair
+ * within 4e-6 of (3h)^2 is decided in FP64, so neighbour sets are those of FP64.  The step order is that of the 2D step (modified
  * Euler predictor, search, volumes, correction tensor, continuity, density filter and equation of
  * state, velocity gradient, Laplacian of Q, Q rate, momentum, artificial displacement, corrector).
  */
@@ -657,8 +658,8 @@ void ann3_destroy(ann3_ctx *c);
 int ann3_set_particles(ann3_ctx *c, int64_t n, const double *x, const double *y, const double *z,
                        const double *u, const double *q, const double *rho);
 
-/* Advance by nsteps steps.  Errors: STATE (no particles), NBR_OVERFLOW, CELL_OVERFLOW,
- * NONFINITE, SINGULAR_ALPHA (sticky device flags set by the kernels' own checks), CUDA. */
+/* Advance by nsteps steps.  Errors: STATE (no particles), NBR_OVERFLOW, NONFINITE, SINGULAR_ALPHA (sticky device flags
+ * set by the kernels' own checks), CUDA. */
 int ann3_step(ann3_ctx *c, int64_t nsteps);
 
 /* A field in ID order into host FP64 dst (n x components, interleaved per particle).  Errors:

@@ -65,7 +65,9 @@ constexpr int MAXC3 = 576;          // candidates: neighbours within 3h (1 + SKI
 constexpr double CELL3 = 0.05;      // cells are at least 3h (1 + CELL3) wide
 constexpr double SPARSE3 = 50.0, GROW3 = 3.0;   // and wider, up to GROW3 times, where they would hold fewer than SPARSE3 particles: see cells3
 // Candidate lists stay valid while no particle moves SKIN3 3h / 2.  A skin of 0.02 keeps ~6 % more
-// candidates than neighbours (0.05: 16 %); a re-sort costs about one step and a half.
+// candidates than neighbours (0.05: 16 %); a re-sort costs about one step and a half.  us a step of 64^3 in a
+// box-scale flow with a re-sort in 180 / 36 / 13 / 4 steps at 0.02: 865 / 885 / 919 / 1,047; with 0.05 (half as many or fewer)
+// 921 / 932 / 943 / 1,004: the smaller skin loses only where every fourth step re-sorts.
 constexpr double SKIN3 = 0.02;
 constexpr uint32_t E3_NBR = 4u, E3_NONFINITE = 8u, E3_ALPHA = 16u;
 

@@ -35,7 +35,7 @@ constexpr int NKERNELS = 10;
 // Candidate ("Verlet") lists hold every pair within 3h (1 + SKIN) at the last re-sort; they stay
 // valid until some particle has moved SKIN/2 * 3h.  Cells are at least 3h (1 + SKIN) wide.
 constexpr double SKIN = 0.02;
-constexpr int MAXV = 128;             // candidates per particle (two 64-bit neighbour masks)
+constexpr int MAXV = 128;             // candidates per particle (32 list words of four)
 constexpr int SCAN_CHUNK = 4096;      // cells per block of the cell-count scan
 
 // Sticky device error bits.

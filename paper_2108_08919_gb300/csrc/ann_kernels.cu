@@ -4,8 +4,8 @@
 // cells are numbered row-major.  A pair pass runs one block per 4 x 4 cells ("tile"): the block
 // stages the particles of the surrounding 6 x 6 cells in shared memory -- periodic images of the
 // cells on the far side of the box take the place of the paper's ghost particles (Eq. 30) -- and
-// each thread accumulates the sums of one particle over its neighbours.  Positions are FP64; the pair
-// passes use a split tile-local coordinate hi + lo in FP32 whose hi parts lie on a power-of-two grid,
+// a thread, or up to eight lanes where the tiles are few, accumulates the sums of one particle over its
+// neighbours.  Positions are FP64; the pair passes use a split tile-local coordinate hi + lo in FP32 whose hi parts lie on a power-of-two grid,
 // so d = (hi_i - hi_j) + (lo_i - lo_j) is the correctly rounded FP32 pair vector.  The support test
 // |d|^2 < (3h)^2 is decided in FP32 unless it falls within a rounding band of the cutoff, where it is
 // redone in FP64 from the FP64 positions exactly as the definition states.
