@@ -29,10 +29,10 @@
 // capacity (dense clusters, boxes of 14 to 16 spacings) reads its candidates from global memory through
 // 32-bit lists instead, in the same kernels.
 //
-// What bounds it (GB300, 64^3, ~250 neighbours): FP32 and issue (the FMA pipe is 45-60 % busy), and the
-// shared-memory loads (60 % of the LSU's cycles; consecutive particles' lists drift apart, so a load
-// takes about twice its least wavefronts).  Filter, pass 1, 2 and 3 take 136, 180, 213 and 314 us; one
-// thread per particle gathering through L1, with lists of the exact neighbours and the
+// What bounds it (GB300, 64^3, ~250 neighbours): FP32 and issue (filter, pass 1, 2, 3: the FMA pipe is busy in 40, 47, 52 and
+// 54 % of cycles, issue in 72, 54, 62 and 62 %), and the shared-memory loads (62, 69, 78 and 70 % of the LSU's data
+// cycles; consecutive particles' lists drift apart, so a load takes about twice its least wavefronts).  They take
+// 140, 190, 211 and 306 us; one thread per particle gathering through L1, with lists of the exact neighbours and the
 // Laplacian as six sums per component in pass 1, took 305, 351, 194 and 335 (predictor: 55, now 18).
 //
 // The state lives in S between steps, in the cell order of the last re-sort.  Errors are sticky bits
