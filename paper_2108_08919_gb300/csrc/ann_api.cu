@@ -1752,8 +1752,8 @@ cudaError_t build_ensemble_graph(ann_ensemble *E, int groups)
         E->exec = nullptr;
     }
     // The wider blocks pay where all tiles run at once, here those of `groups` members side by side: 64
-    // members of 128^2 to 512^2 take 2.98 ms a step in 16 branches and in 64 with 256 threads, 3.07 and 3.10
-    // with 288.  A particle's sums are the same either way, so members stay bit-identical to solo runs.
+    // members of 128^2 to 512^2 took 2.98 ms a step in 16 branches and in 64 with 256 threads, 3.07 and 3.10
+    // with 288 (2.90 now that members of several lanes take them in turn).  A particle's sums are the same either way, so members stay bit-identical to solo runs.
     const int64_t members = (int64_t)E->m.size();
     int64_t tiles = 0, mean = 0;
     for (const ann_ctx *c : E->m) {
